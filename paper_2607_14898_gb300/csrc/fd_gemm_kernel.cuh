@@ -3,8 +3,8 @@
 // A: bf16 [M][K] row-major (activations), W: bf16 [N][K] row-major (nn.Linear weight), both
 // K-major, loaded by TMA with the 128-byte swizzle into a ring of shared-memory stages.
 // One persistent CTA per SM walks 128 x BN output tiles. Warp roles:
-//   warp 0 (one lane)  TMA producer: stages of 128x64 (A) and BNx64 (W)
-//   warp 1 (one lane)  MMA issuer: 4 x tcgen05.mma (K = 16 each) per stage into a TMEM
+//   warp 0             TMA producer: stages of 128x64 (A) and BNx64 (W)
+//   warp 1             MMA issuer: 4 x tcgen05.mma (K = 16 each) per stage into a TMEM
 //                      accumulator; two accumulators so the epilogue of tile i overlaps the
 //                      MMAs of tile i+1
 //   warps 2-5          epilogue: each thread owns one accumulator row (TMEM lane), applies
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(192, 1)
   constexpr int kTmemCols = DS ? 4 * BN : C::kTmemCols;
   static_assert(!DS || (!PAIR && QKV == 0 && 4 * BN <= 512), "scores backward: single CTAs");
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_index();
   const int lane = threadIdx.x & 31;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kBarOffset);
   const uint32_t bar_full = smem_u32(bars);                    // [kStages]
@@ -197,16 +197,19 @@ __global__ void __launch_bounds__(192, 1)
   }
   if (PAIR) cluster_sync();  // both CTAs' barriers exist before any load or commit reaches them
   // Weights that no kernel of the stream writes (p.w_static) are loaded into the first stages
-  // while the previous kernel is still finishing; only the activations wait for it. Thread 0
-  // is the TMA producer and initialised the barriers above.
+  // while the previous kernel is still finishing; only the activations wait for it. Warp 0 is the
+  // TMA producer and its thread 0 initialised the barriers above.
   const int pre = (p.w_static && aligned && cta0 < tiles)
                       ? (nk < C::kStages ? nk : C::kStages)
                       : 0;
-  if (threadIdx.x == 0) {
+  if (warp == 0) {
+    __syncwarp();
     const int nb0 = (cta0 % n_tiles) * BN + static_cast<int>(rank) * C::kBRows;
     for (int kb = 0; kb < pre; ++kb) {
-      if (rank == 0) mbar_expect_tx(bar_full + 8 * kb, full_tx);
-      load(sB + kb * C::kBBytes, &tmB, kb, kb * kel, nb0);
+      if (elect_one()) {
+        if (rank == 0) mbar_expect_tx(bar_full + 8 * kb, full_tx);
+        load(sB + kb * C::kBBytes, &tmB, kb, kb * kel, nb0);
+      }
     }
   }
   grid_dep_wait();  // inputs written by the previous kernel; TMEM freed by its CTAs
@@ -222,10 +225,11 @@ __global__ void __launch_bounds__(192, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
-  if (aligned && warp == 0 && lane == 0) {
+  if (aligned && warp == 0) {
     // ------------------------------------------------------------ TMA producer
+    // (the whole warp runs the loop; one elected lane issues)
     int it = 0;
     bool ok = true;
     for (int tile = cta0; tile < tiles && ok; tile += ctas) {
@@ -235,27 +239,31 @@ __global__ void __launch_bounds__(192, 1)
         const int s = it % C::kStages;
         const uint32_t ph = (it / C::kStages) & 1;
         if (it < pre) {  // W already on its way: the activation half of the stage
-          load(sA + s * C::kABytes, &tmA, s, kb * kel, m0);
+          if (elect_one()) load(sA + s * C::kABytes, &tmA, s, kb * kel, m0);
           continue;
         }
-        if (!mbar_wait(bar_empty + 8 * s, ph ^ 1, p.err, ERR_WAIT_MMA)) { ok = false; break; }
-        if (rank == 0) mbar_expect_tx(bar_full + 8 * s, full_tx);
-        if (DS) {  // block 0: Q and K; block 1: dO and V (K = 64, one block each)
-          load(sA + s * C::kABytes, kb == 0 ? &tmA : &tmK, s, 0, m0);
-          load(sB + s * C::kBBytes, kb == 0 ? &tmB : &tmV, s, 0, nb0);
-          continue;
+        if (!mbar_wait_warp(bar_empty + 8 * s, ph ^ 1, p.err, ERR_WAIT_MMA)) { ok = false; break; }
+        if (elect_one()) {
+          if (rank == 0) mbar_expect_tx(bar_full + 8 * s, full_tx);
+          if (DS) {  // block 0: Q and K; block 1: dO and V (K = 64, one block each)
+            load(sA + s * C::kABytes, kb == 0 ? &tmA : &tmK, s, 0, m0);
+            load(sB + s * C::kBBytes, kb == 0 ? &tmB : &tmV, s, 0, nb0);
+          } else {
+            load(sA + s * C::kABytes, &tmA, s, kb * kel, m0);
+            load(sB + s * C::kBBytes, &tmB, s, kb * kel, nb0);
+          }
         }
-        load(sA + s * C::kABytes, &tmA, s, kb * kel, m0);
-        load(sB + s * C::kBBytes, &tmB, s, kb * kel, nb0);
       }
     }
     // drain: the loads issued last must land before the CTA may exit (pairs: they have once
     // rank 0's MMAs have read their stages, which releases the stage in both CTAs)
     for (int j = it - 1; j >= 0 && j >= it - C::kStages; --j) {
       if (PAIR)
-        mbar_wait(bar_empty + 8 * (j % C::kStages), (j / C::kStages) & 1, p.err, ERR_WAIT_MMA);
+        mbar_wait_warp(bar_empty + 8 * (j % C::kStages), (j / C::kStages) & 1, p.err,
+                       ERR_WAIT_MMA);
       else
-        mbar_wait(bar_full + 8 * (j % C::kStages), (j / C::kStages) & 1, p.err, ERR_WAIT_TMA);
+        mbar_wait_warp(bar_full + 8 * (j % C::kStages), (j / C::kStages) & 1, p.err,
+                       ERR_WAIT_TMA);
     }
   } else if (aligned && warp == 1 && rank == 0) {
     // ------------------------------------------------------------ MMA issuer

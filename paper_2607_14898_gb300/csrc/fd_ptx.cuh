@@ -116,6 +116,25 @@ __device__ __forceinline__ void prefetch_l1(const void* p) {
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
 }
+// true in one lane of a converged warp (the same lane every time). Single-thread instructions
+// (TMA, MMA, mbarrier arrives) sit in `if (elect_one())` inside code the whole warp runs, with a
+// warp index from warp_index(): the compiler then keeps their operands in uniform registers. A
+// lane picked by `lane == 0` in a branch on threadIdx pays a move into them for each operand:
+// a producer of two tile loads per stage took 401 cycles a stage that way (any tile size, any
+// number of stages), 246 this way at 128 x 96 tiles, where the SM's intake of ~118 bytes a
+// clock is the limit.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t"
+      "elect.sync r|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
+}
+// this thread's warp, as a value the compiler knows to be the same in the whole warp
+__device__ __forceinline__ int warp_index() {
+  return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
+}
 // 2D tile load, x = innermost coordinate (elements), y = row; completes on `bar`.
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* m, uint32_t bar,
                                             int x, int y) {
