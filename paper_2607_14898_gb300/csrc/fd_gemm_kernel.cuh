@@ -7,11 +7,12 @@
 //   warp 1             MMA issuer: 4 x tcgen05.mma (K = 16 each) per stage into a TMEM
 //                      accumulator; two accumulators so the epilogue of tile i overlaps the
 //                      MMAs of tile i+1
-//   warps 2-5          epilogue: each thread owns one accumulator row (TMEM lane), applies
-//                      the fused epilogue, and writes its row of a 32-row slab into a
-//                      128-byte-swizzled staging buffer; one lane then stores the slab with a
-//                      TMA bulk tensor store (a bulk reduce-add for the residual), so global
-//                      writes are whole lines and rows past M are clipped by the tensor map
+//   warps 2-9 (QKV: 2-5) epilogue, two warps (one) per 32 accumulator rows (TMEM lanes), taking
+//                      the tile's column chunks in turn: each thread owns one row, applies the fused
+//                      epilogue, and writes its row of a 32-row slab into a swizzled staging
+//                      buffer; one lane then stores the slab with a TMA bulk tensor store (a
+//                      bulk reduce-add for the residual), so global writes are whole lines (or
+//                      halves) and rows past M are clipped by the tensor map
 // Fused epilogues (the linear layers of Sec. 3.2 / 3.4 and Eq. projection / temporal_upsample):
 //   EPI_F32    out = acc + b                    (patch-embed, head layer 2)
 //   EPI_RESID  h  += acc + b                    (out-projection, MLP layer 2: residual)
@@ -39,22 +40,35 @@
 
 namespace fd {
 
+// Epilogue warps: eight (two per 32 accumulator rows, alternate column chunks). With four, the
+// GELU and SwiGLU epilogues took longer than the tile's MMAs at K = 1024, and every product paid
+// its last tile's epilogue at half the speed: refinement MLP1 (6240 x 4096 x 1024) 45.7 -> 39.7
+// us, e4m3 GELU (1560 x 4096 x 1024) 18.6 -> 11.2, batched MLP1 (13312 rows) 80 -> 69. The QKV
+// epilogue keeps four: it computes each row's rotation once per warp, and two warps per row
+// measured slower (480p QKV 10.4 -> 12.0).
+constexpr int epi_warps(int qkv) { return qkv ? 4 : 8; }
+
 // PAIR: the tile is 256 x BN, computed by a cluster of two CTAs with tcgen05 cta_group::2
 // MMAs issued by the even CTA: each CTA holds its 128 rows of A and half (BN/2 rows) of W per
 // stage, the pair's tensor cores read both halves, and each CTA's TMEM receives its 128 rows of
 // the accumulator. Per SM, a stage then needs 16 KB + 64 BN bytes for 2 BN MMA cycles instead of
 // 16 KB + 128 BN, which is what bounds the single-CTA kernel (shared-memory intake per SM).
-template <int BN, bool PAIR>
+template <int BN, bool PAIR, int QKV>
 struct GemmCfg {
+  static constexpr int kEpiWarps = epi_warps(QKV);
+  static constexpr int kThreads = 64 + 32 * kEpiWarps;
   static constexpr int kABytes = kBM * kBK * 2;  // 16 KB
   static constexpr int kBRows = PAIR ? BN / 2 : BN;
   static constexpr int kBBytes = kBRows * kBK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kRoom = (227 * 1024 - 4 * 2 * 4096 - 256) / kStageBytes;
-  static constexpr int kStages = PAIR ? (kRoom > 8 ? 8 : kRoom) : (BN >= 192 ? 4 : 6);
+  // one 4 KB staging buffer per epilogue warp: the other warp of the scheduler works while a
+  // store reads it, and a second one would cost the pipeline a stage
+  static constexpr int kStgBytes = kEpiWarps * 4096;
+  static constexpr int kRoom = (227 * 1024 - kStgBytes - 256) / kStageBytes;
+  static constexpr int kStages = kRoom > (PAIR ? 8 : 6) ? (PAIR ? 8 : 6) : kRoom;
   static constexpr int kTmemCols = 2 * BN <= 128 ? 128 : (2 * BN <= 256 ? 256 : 512);
-  static constexpr int kStgOffset = kStages * kStageBytes;   // 4 warps x 2 x 4 KB staging
-  static constexpr int kBarOffset = kStgOffset + 4 * 2 * 4096;
+  static constexpr int kStgOffset = kStages * kStageBytes;
+  static constexpr int kBarOffset = kStgOffset + kStgBytes;
   static constexpr int kSmem = kBarOffset + 256;
   static_assert(kSmem <= 227 * 1024, "shared memory");
   static_assert((kBRows * 128) % 1024 == 0, "W stages start on a swizzle atom");
@@ -65,6 +79,13 @@ __device__ __forceinline__ void put_row_sw128(uint8_t* buf, int row, const uint3
 #pragma unroll
   for (int k = 0; k < 8; ++k)
     *reinterpret_cast<uint4*>(buf + row * 128 + ((k ^ (row & 7)) << 4)) =
+        make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+}
+// the same for a 64-byte row (4 x 16 B) in the 64-byte-swizzled layout
+__device__ __forceinline__ void put_row_sw64(uint8_t* buf, int row, const uint32_t* w) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    *reinterpret_cast<uint4*>(buf + row * 64 + ((k ^ ((row >> 1) & 3)) << 4)) =
         make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
 }
 
@@ -138,11 +159,11 @@ __device__ __forceinline__ void rope_table(const QkvEpi& q, const float2* rope_t
 // exp(S scale - lse) (p.ds), written as dS rows and dS^T, P^T columns (bf16). S and dP are never
 // stored.
 template <int BN, bool PAIR, int QKV, bool DS = false>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ GemmParams p) {
-  using C = GemmCfg<BN, PAIR>;
+  using C = GemmCfg<BN, PAIR, QKV>;
   // accumulator columns of one tile (DS: S and dP side by side), two tiles in flight
   constexpr uint32_t kAccCols = DS ? 2 * BN : BN;
   constexpr int kTmemCols = DS ? 4 * BN : C::kTmemCols;
@@ -188,7 +209,7 @@ __global__ void __launch_bounds__(192, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(bar_tfull + 8 * a, 1);
-      mbar_init(bar_tempty + 8 * a, PAIR ? 8 : 128);  // pairs: one arrive per epilogue warp
+      mbar_init(bar_tempty + 8 * a, PAIR ? 2 * C::kEpiWarps : C::kEpiWarps);  // one arrive per warp
     }
     mbar_init(bar_done, 1);
     fence_barrier_init();
@@ -315,16 +336,16 @@ __global__ void __launch_bounds__(192, 1)
   } else if (aligned && warp >= 2) {
     // ------------------------------------------------------------ epilogue
     const int quarter = warp & 3;  // TMEM lanes this warp may read
+    constexpr int kHalves = C::kEpiWarps / 4;  // warps per 32 rows
+    const int half = (warp - 2) >> 2;          // this one's chunks: half, half + kHalves, ...
     const int rloc = quarter * 32 + lane;
-    uint8_t* stg = smem + C::kStgOffset + (warp - 2) * 8192;
-    int sb = 0;
-    // a free 4 KB staging buffer: the store issued from it two stores ago has read it
+    uint8_t* const stg = smem + C::kStgOffset + (warp - 2) * 4096;
+    // the warp's staging buffer, once the store issued from it has read it (stores are issued,
+    // committed and waited for by the elected lane)
     auto acquire = [&]() -> uint8_t* {
-      if (lane == 0) bulk_wait_read_1();
+      if (elect_one()) bulk_wait_read_0();
       __syncwarp();
-      uint8_t* b = stg + sb * 4096;
-      sb ^= 1;
-      return b;
+      return stg;
     };
     auto publish = [&]() {  // make the slab visible to the TMA engine
       fence_proxy_async_smem();
@@ -403,7 +424,7 @@ __global__ void __launch_bounds__(192, 1)
         // MMAs of the tile still run
         if (!acc_ready()) break;
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 64) {
+        for (int c = 64 * half; c < BN; c += 64 * kHalves) {
           const int col = n0 + c;
           if (col >= p.N) break;  // warp-uniform
           uint32_t r0[32], r1[32];
@@ -458,7 +479,7 @@ __global__ void __launch_bounds__(192, 1)
             uint8_t* buf = acquire();
             put_row_sw128(buf, lane, w);
             publish();
-            if (lane == 0 && row0 < p.M) {  // a slab wholly past M stores nothing
+            if (row0 < p.M && elect_one()) {  // a slab wholly past M stores nothing
               if (is_q) {
                 tma_store_2d(&tmO, smem_u32(buf), hidx * kHeadDim, row0);
               } else {
@@ -473,7 +494,7 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll
             for (int j = 0; j < 64; ++j) sv[j * 32 + lane] = __float2half_rn(v[j]);
             publish();
-            if (lane == 0 && row0 < p.M) {
+            if (row0 < p.M && elect_one()) {
               tma_store_4d(&tmV, smem_u32(buf), row0, slot, 0, hidx - q.heads - q.groups);
               bulk_commit();
             }
@@ -494,7 +515,7 @@ __global__ void __launch_bounds__(192, 1)
         const float lse = row_ok ? __ldg(q.lse + row) : 0.f;
         const float dlt = row_ok ? __ldg(q.delta + row) : 0.f;
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
+        for (int c = 32 * half; c < BN; c += 32 * kHalves) {
           const int col = n0 + c;
           if (col >= p.N) break;  // N % 32 == 0
           uint32_t rs[32], rp[32];
@@ -529,7 +550,7 @@ __global__ void __launch_bounds__(192, 1)
         }
       } else if (p.epi == EPI_GELU) {
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 64) {
+        for (int c = 64 * half; c < BN; c += 64 * kHalves) {
           const int col = n0 + c;
           if (col >= p.N) break;
           uint32_t r0[32], r1[32];
@@ -553,25 +574,25 @@ __global__ void __launch_bounds__(192, 1)
           uint8_t* buf = acquire();
           put_row_sw128(buf, lane, w);
           publish();
-          if (lane == 0 && row0 < p.M) {
+          if (row0 < p.M && elect_one()) {
             tma_store_2d(&tmO, smem_u32(buf), col, row0);
             bulk_commit();
           }
         }
       } else if (p.epi == EPI_GELU_F8) {
-        // 128 accumulator columns -> one 128-byte row of e4m3 per slab
+        // 64 accumulator columns -> one 64-byte row of e4m3 per slab
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 128) {
+        for (int c = 64 * half; c < BN; c += 64 * kHalves) {
           const int col = n0 + c;
           if (col >= p.N) break;
-          uint32_t w[32];
+          uint32_t w[16];
 #pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
+          for (int q2 = 0; q2 < 2; ++q2) {
             uint32_t r[32];
             __syncwarp();
-            tmem_ld_32x32b_x32(tbase + c + 32 * q4, r);
+            tmem_ld_32x32b_x32(tbase + c + 32 * q2, r);
             tmem_ld_wait();
-            const int cb = col + 32 * q4;
+            const int cb = col + 32 * q2;
             float cs[32], bb[32];
             load32(p.col_scale + cb, cs);
             load32(p.bias + cb, bb);
@@ -582,26 +603,26 @@ __global__ void __launch_bounds__(192, 1)
               for (int e = 0; e < 4; ++e)
                 f[e] = gelu_erf(fmaf(__uint_as_float(r[4 * j + e]), cs[4 * j + e], bb[4 * j + e])) *
                        p.out_scale;
-              w[8 * q4 + j] = pack_e4m3x4(f[0], f[1], f[2], f[3]);
+              w[8 * q2 + j] = pack_e4m3x4(f[0], f[1], f[2], f[3]);
             }
           }
           uint8_t* buf = acquire();
-          put_row_sw128(buf, lane, w);
+          put_row_sw64(buf, lane, w);
           publish();
-          if (lane == 0 && row0 < p.M) {
+          if (row0 < p.M && elect_one()) {
             tma_store_2d(&tmO, smem_u32(buf), col, row0);
             bulk_commit();
           }
         }
       } else if (p.epi == EPI_SWIGLU_F8) {
-        // 256 accumulator columns (4 blocks of 32 gate + 32 up) -> one 128-byte e4m3 row
+        // 128 accumulator columns (2 blocks of 32 gate + 32 up) -> one 64-byte e4m3 row
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 256) {
+        for (int c = 128 * half; c < BN; c += 128 * kHalves) {
           const int col = n0 + c;
           if (col >= p.N) break;
-          uint32_t w[32];
+          uint32_t w[16];
 #pragma unroll
-          for (int hh = 0; hh < 4; ++hh) {
+          for (int hh = 0; hh < 2; ++hh) {
             uint32_t rg[32], ru[32];
             __syncwarp();
             tmem_ld_32x32b_x32(tbase + c + 64 * hh, rg);
@@ -626,42 +647,42 @@ __global__ void __launch_bounds__(192, 1)
               w[8 * hh + j] = pack_e4m3x4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
           }
           uint8_t* buf = acquire();
-          put_row_sw128(buf, lane, w);
+          put_row_sw64(buf, lane, w);
           publish();
-          if (lane == 0 && row0 < p.M) {
+          if (row0 < p.M && elect_one()) {
             tma_store_2d(&tmO, smem_u32(buf), col / 2, row0);
             bulk_commit();
           }
         }
       } else if (p.epi == EPI_SWIGLU) {
+        // 64 accumulator columns (32 gate + 32 up) -> one 64-byte bf16 row
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 128) {
+        for (int c = 64 * half; c < BN; c += 64 * kHalves) {
           const int col = n0 + c;
           if (col >= p.N) break;
-          uint32_t w[32];
-#pragma unroll
-          for (int hh = 0; hh < 2; ++hh) {
-            uint32_t rg[32], ru[32];
-            __syncwarp();
-            tmem_ld_32x32b_x32(tbase + c + 64 * hh, rg);
-            tmem_ld_32x32b_x32(tbase + c + 64 * hh + 32, ru);
-            tmem_ld_wait();
+          uint32_t rg[32], ru[32];
+          __syncwarp();
+          tmem_ld_32x32b_x32(tbase + c, rg);
+          tmem_ld_32x32b_x32(tbase + c + 32, ru);
+          tmem_ld_wait();
+          uint32_t w[16];
+          {
             float bgv[32], buv[32];
-            load32(p.bias + col + 64 * hh, bgv);
-            load32(p.bias + col + 64 * hh + 32, buv);
+            load32(p.bias + col, bgv);
+            load32(p.bias + col + 32, buv);
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               const float g0 = __uint_as_float(rg[2 * j]) + bgv[2 * j];
               const float g1 = __uint_as_float(rg[2 * j + 1]) + bgv[2 * j + 1];
               const float u0 = __uint_as_float(ru[2 * j]) + buv[2 * j];
               const float u1 = __uint_as_float(ru[2 * j + 1]) + buv[2 * j + 1];
-              w[16 * hh + j] = pack_bf16x2(silu(g0) * u0, silu(g1) * u1);
+              w[j] = pack_bf16x2(silu(g0) * u0, silu(g1) * u1);
             }
           }
           uint8_t* buf = acquire();
-          put_row_sw128(buf, lane, w);
+          put_row_sw64(buf, lane, w);
           publish();
-          if (lane == 0 && row0 < p.M) {
+          if (row0 < p.M && elect_one()) {
             tma_store_2d(&tmO, smem_u32(buf), col / 2, row0);
             bulk_commit();
           }
@@ -675,7 +696,7 @@ __global__ void __launch_bounds__(192, 1)
         const int gy = l / px.gw, gx = l - gy * px.gw;
         const int rs = px.rs, rs2 = rs * rs, Wo = px.gw * rs, Ho = px.gh * rs;
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
+        for (int c = 32 * half; c < BN; c += 32 * kHalves) {
           const int col = n0 + c;
           if (col >= p.N) break;
           uint32_t r[32];
@@ -707,7 +728,7 @@ __global__ void __launch_bounds__(192, 1)
         }
       } else {  // EPI_F32, EPI_RESID, EPI_TUP: fp32 slabs of 32 columns
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
+        for (int c = 32 * half; c < BN; c += 32 * kHalves) {
           const int col = n0 + c;
           if (col >= p.N) break;
           uint32_t r[32];
@@ -730,7 +751,7 @@ __global__ void __launch_bounds__(192, 1)
           uint8_t* buf = acquire();
           put_row_sw128(buf, lane, w);
           publish();
-          if (lane == 0 && row0 < p.M) {
+          if (row0 < p.M && elect_one()) {
             if (p.epi == EPI_RESID) {
               tma_reduce_add_2d(&tmO, smem_u32(buf), col, row0);
             } else if (p.epi == EPI_TUP) {
@@ -745,15 +766,16 @@ __global__ void __launch_bounds__(192, 1)
           }
         }
       }
-      __syncwarp();
       tc_fence_before();
-      if (PAIR) {  // one arrive per warp on rank 0's barrier
-        if (lane == 0) mbar_arrive_remote(bar_tempty0 + 8 * acc);
-      } else {
-        mbar_arrive(bar_tempty + 8 * acc);
+      __syncwarp();
+      if (elect_one()) {  // one arrive per warp (pairs: on rank 0's barrier)
+        if (PAIR) mbar_arrive_remote(bar_tempty0 + 8 * acc);
+        else mbar_arrive(bar_tempty + 8 * acc);
       }
     }
-    if (lane == 0) bulk_wait_all();  // every store has landed before the CTA exits
+    // every store has read its buffer before the CTA exits (its writes complete with the grid,
+    // which is what a dependent kernel's griddepcontrol.wait waits for)
+    if (elect_one()) bulk_wait_read_0();
     __syncwarp();
   }
   grid_dep_launch();
@@ -773,14 +795,14 @@ static cudaError_t launch_bn(const CUtensorMap& tmA, const CUtensorMap& tmB,
                              const CUtensorMap& tmO, const CUtensorMap& tmK,
                              const CUtensorMap& tmV, const GemmParams& p, int num_sms,
                              cudaStream_t s) {
-  using C = GemmCfg<BN, PAIR>;
+  using C = GemmCfg<BN, PAIR, QKV>;
   static const cudaError_t attr = cudaFuncSetAttribute(
       gemm_kernel<BN, PAIR, QKV, DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
   if (attr != cudaSuccess) return attr;
   const int rows = PAIR ? 2 * kBM : kBM;
   const int tiles = ((p.M + rows - 1) / rows) * ((p.N + BN - 1) / BN);
   cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(192);
+  cfg.blockDim = dim3(C::kThreads);
   cfg.dynamicSmemBytes = C::kSmem;
   cfg.stream = s;
   cudaLaunchAttribute at[2];

@@ -110,6 +110,8 @@ struct QkvEpi {
 // are 32-row slabs, 128-byte swizzled unless noted):
 //   EPI_F32 / EPI_RESID  tmO: fp32 [M][ld_out], box {32, 32} (RESID uses a bulk reduce-add)
 //   EPI_GELU             tmO: bf16 [M][ld_out], box {64, 32}
+//   EPI_SWIGLU           tmO: bf16 [M][ld_out], box {32, 32}, 64-byte swizzle
+//   EPI_*_F8             tmO: e4m3 [M][ld_out], box {64, 32}, 64-byte swizzle
 //   EPI_TUP              tmO: fp32 3D {D, L, r_t}, box {32, 32, 1}
 //   EPI_QKV              tmO: Q bf16 [M][heads*64], box {64, 32};
 //                        tmK: K ring 4D {64, M, W, G} (row, slot, group strides), box {64,32,1,1};

@@ -94,9 +94,9 @@ bool tmap_e4m3(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer,
 // GEMM epilogue store maps (32-row slabs)
 bool tmap_out_e4m3(CUtensorMap* m, const void* base, uint64_t cols, uint64_t rows, uint64_t ld) {
   const uint64_t dims[2] = {cols, rows}, strides[1] = {ld};
-  const uint32_t box[2] = {128, 32};
+  const uint32_t box[2] = {64, 32};
   return tmap_nd(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box,
-                 CU_TENSOR_MAP_SWIZZLE_128B);
+                 CU_TENSOR_MAP_SWIZZLE_64B);
 }
 bool tmap_out_f32(CUtensorMap* m, const void* base, uint64_t cols, uint64_t rows, uint64_t ld) {
   const uint64_t dims[2] = {cols, rows}, strides[1] = {ld * 4};
@@ -109,6 +109,13 @@ bool tmap_out_bf16(CUtensorMap* m, const void* base, uint64_t cols, uint64_t row
   const uint32_t box[2] = {64, 32};
   return tmap_nd(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box,
                  CU_TENSOR_MAP_SWIZZLE_128B);
+}
+// the gated epilogue's bf16 output: 64 accumulator columns give 32 values, a 64-byte row
+bool tmap_out_gated(CUtensorMap* m, const void* base, uint64_t cols, uint64_t rows, uint64_t ld) {
+  const uint64_t dims[2] = {cols, rows}, strides[1] = {ld * 2};
+  const uint32_t box[2] = {32, 32};
+  return tmap_nd(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box,
+                 CU_TENSOR_MAP_SWIZZLE_64B);
 }
 // temporal upsampling output viewed as [streams][r_t][L][D] (L rows per refined frame)
 bool tmap_out_tup(CUtensorMap* m, const void* base, uint64_t D, uint64_t L, uint64_t rt,
@@ -1430,8 +1437,9 @@ fd_status fd_create(const fd_config* cfg, fd_weights w, fd_handle* out) {
   ok = ok && tmap_out_f32(&h->so_h, h->h, d.D, d.L, d.D);
   ok = ok && tmap_out_f32(&h->so_hf, h->hf, d.D, R, d.D);
   ok = ok && tmap_out_tup(&h->so_tup, h->hf, d.D, d.L, d.rt);
-  ok = ok && tmap_out_bf16(&h->so_hidB, h->hid, Dm, d.L, Dm);
-  ok = ok && tmap_out_bf16(&h->so_hidR, h->hid, Dm, R, Dm);
+  const auto tmap_hid = d.gated ? tmap_out_gated : tmap_out_bf16;
+  ok = ok && tmap_hid(&h->so_hidB, h->hid, Dm, d.L, Dm);
+  ok = ok && tmap_hid(&h->so_hidR, h->hid, Dm, R, Dm);
   ok = ok && tmap_out_bf16(&h->so_hidH, h->hid, d.D, R, d.D);
   ok = ok && tmap_out_f32(&h->so_F, h->F, d.head_out, R, d.head_out);
   ok = ok && tmap_out_bf16(&h->so_qB, h->q, NQ, d.L, NQ);
@@ -1610,8 +1618,9 @@ fd_status fd_batch_create(const fd_config* cfg, fd_weights w, int max_streams, f
   ok = ok && tmap_out_f32(&b->so_h, b->h, d.D, RB, d.D);
   ok = ok && tmap_out_f32(&b->so_hf, b->hf, d.D, RR, d.D);
   ok = ok && tmap_out_tup(&b->so_tup, b->hf, d.D, b->Lp, d.rt, max_streams);
-  ok = ok && tmap_out_bf16(&b->so_hidB, b->hid, Dm, RB, Dm);
-  ok = ok && tmap_out_bf16(&b->so_hidR, b->hid, Dm, RR, Dm);
+  const auto tmap_hid = d.gated ? tmap_out_gated : tmap_out_bf16;
+  ok = ok && tmap_hid(&b->so_hidB, b->hid, Dm, RB, Dm);
+  ok = ok && tmap_hid(&b->so_hidR, b->hid, Dm, RR, Dm);
   ok = ok && tmap_out_bf16(&b->so_hidH, b->hid, d.D, RR, d.D);
   ok = ok && tmap_out_f32(&b->so_F, b->F, d.head_out, RR, d.head_out);
   ok = ok && tmap_out_bf16(&b->so_qB, b->q, NQ, RB, NQ);
@@ -2078,7 +2087,7 @@ fd_status fd_op_linear_tiled(int epilogue, int M, int N, int K, const void* A, c
   CUtensorMap to;
   bool ok;
   if (epilogue == FD_EPI_GELU) ok = tmap_out_bf16(&to, out, N, M, N);
-  else if (epilogue == FD_EPI_SWIGLU) ok = tmap_out_bf16(&to, out, N / 2, M, N / 2);
+  else if (epilogue == FD_EPI_SWIGLU) ok = tmap_out_gated(&to, out, N / 2, M, N / 2);
   else if (epilogue == FD_EPI_TUP) ok = tmap_out_tup(&to, out, tup_hidden, M, N / tup_hidden);
   else ok = tmap_out_f32(&to, out, N, M, N);
   if (!ok) return FD_ERR_CUDA;
