@@ -185,6 +185,17 @@ struct AttnParams {
   int lse_pitch;
 };
 
+// Backward of the band attention over a clip of T query chunks (fd_attn_bwd.cu): rows of q / dO
+// [T][N][Pc], Pc = frames x Lp rows per chunk and head (the first L of each Lp are tokens), keys
+// [G][M] with M = T Pc; query chunk i sees key chunks max(0, i - W + 1) .. i. lse of a padding row
+// is +inf. dK and dV sum hs heads of a chunk per accumulator chain.
+struct AttnBwdParams {
+  const float *lse, *delta;  // [T][N][Pc]
+  float *out0, *out1;        // set by the launch
+  int T, N, G, W, Pc, Lp, L, M, hs;
+  int* err;
+};
+
 // launch wrappers; return cudaGetLastError() of the launch
 // pair: 256-row tiles computed by CTA pairs (cta_group::2; bn 96 / 128 / 192 / 256): tmA
 // boxes of 128 rows as for single CTAs, tmB boxes of bn / 2 rows (each CTA loads half of W)
@@ -231,6 +242,11 @@ inline void attention_workspace_split(float* ws, int parts, int pairs, AttnParam
   a.part_o = ws ? ws + attention_counter_floats(pairs) : nullptr;
   a.part_ml = ws ? a.part_o + static_cast<size_t>(parts) * 4 * 64 * 128 : nullptr;
 }
+// dq fp32 [T N Pc][64], dk / dv fp32 [G M][64]; maps of q2, dO [T N Pc][64] and k2, v1 [G M][64]
+// (bf16, boxes of 64 x 128 rows)
+cudaError_t launch_attention_bwd(const CUtensorMap& tmQ, const CUtensorMap& tmdO,
+                                 const CUtensorMap& tmK, const CUtensorMap& tmV, AttnBwdParams p,
+                                 float* dq, float* dk, float* dv, cudaStream_t s);
 cudaError_t launch_unshuffle(const float* z, int C, int H, int W, int p, __nv_bfloat16* x0,
                              cudaStream_t s);
 cudaError_t launch_rmsnorm(const float* h, const float* g, int M, int D, float eps,
@@ -273,6 +289,10 @@ cudaError_t gemm_view(int epi, int M, int N, int K, const __nv_bfloat16* A, int 
 cudaError_t scores_bwd(int M, int N, const __nv_bfloat16* Q, const __nv_bfloat16* dO, int ldq,
                        const __nv_bfloat16* K, const __nv_bfloat16* V, int ldk, const DsEpi& ds,
                        int* err, cudaStream_t s);
+// the same launch with its maps made from the tensors' addresses
+cudaError_t attention_bwd(const __nv_bfloat16* q, const __nv_bfloat16* dO, const __nv_bfloat16* k,
+                          const __nv_bfloat16* v, const AttnBwdParams& p, float* dq, float* dk,
+                          float* dv, cudaStream_t s);
 // Band attention of the training step on the batched attention kernel, one "stream" per query
 // chunk i: its keys are chunks max(0, i - W + 1) .. i of unpadded K bf16 [G][pitch][64] and
 // V^T fp16 [G][64][pitch] (rows_per_chunk keys per chunk), so stream i's maps start at key

@@ -12,13 +12,11 @@
 //     (gemm_view);
 //   - the attention forward: the decode's batched attention kernel with one stream per query
 //     chunk over the window of its key chunks, writing each row's log-sum-exp (attn_fwd);
-//   - the attention backward per (query chunk, KV group): one launch for S = Q K^T and
-//     dP = dO V^T with the softmax derivative dS = P (dP - rowsum(dO O)) in its epilogue
-//     (scores_bwd: S and dP stay in tensor memory), then dQ = dS K, dK += dS^T Q, dV += P^T dO
-//     on the GEMM (attn_bwd).
+//   - the attention backward (fd_attn_bwd.cu): two launches that recompute S = Q K^T and dP =
+//     dO V^T on chip, one for dQ, one for dK and dV.
 // Row-wise and element-wise steps (RMSNorm and its backward, KV-norm / QK-norm with 3D-RoPE and
-// their backward, GELU and GELU', rowsum(dO O), the L1 term through the pixel shuffle, bias and
-// gain sums) are the kernels below. Where a stack's keys per chunk are not a multiple of 8, its
+// their backward, GELU and GELU', the attention backward's operands, the L1 term through the
+// pixel shuffle, bias and gain sums) are the kernels below. Where a stack's keys per chunk are not a multiple of 8, its
 // attention forward is materialised instead (S, the band softmax, O = P V).
 //
 // Rows: chunk c's L tokens sit at rows c Lp .. c Lp + L - 1 with Lp = 128 ceil(L / 128), the
@@ -398,36 +396,42 @@ __global__ void softmax_lse_kernel(const float* __restrict__ S, int rows, int n,
   if (lane == 0) lse[row] = l;
 }
 
-// delta[(c N + h) Pc + l] = sum_j dO[c Pc + l][h 64 + j] O[c Pc + l][h 64 + j]: dO fp32 and
-// O bf16, both rows [M][N 64]; one warp per (chunk, head, row)
-__global__ void delta_kernel(const float* __restrict__ dO, const bf16* __restrict__ O, int M,
-                             int Pc, int N, float* __restrict__ delta) {
+// Operands of the attention backward from dO fp32 rows [M][N 64], one warp per (row, head): dO
+// head-major bf16 [M / Pc][N][Pc][64], delta[(c N + h) Pc + l] = sum_j dO O of the row and head
+// (O bf16 rows), and lse of padding rows set to +inf (their P is then exp(-inf) = 0)
+__global__ void attn_bwd_prep_kernel(const float* __restrict__ dO, const bf16* __restrict__ O,
+                                     int M, int Pc, int Lp, int L, int N, bf16* __restrict__ do16,
+                                     float* __restrict__ delta, float* __restrict__ lse) {
   const long long w = (blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= static_cast<long long>(M) * N) return;
-  const int c = static_cast<int>(w / (static_cast<long long>(N) * Pc));
-  const int h = static_cast<int>(w / Pc % N), l = static_cast<int>(w % Pc);
-  const size_t e = (static_cast<size_t>(c) * Pc + l) * N * kDh + h * kDh;
+  const int m = static_cast<int>(w / N), h = static_cast<int>(w % N);
+  const size_t e = (static_cast<size_t>(m) * N + h) * kDh;
   const float* a = dO + e;
   const bf16* b = O + e;
-  float v = a[lane] * __bfloat162float(b[lane]) + a[lane + 32] * __bfloat162float(b[lane + 32]);
+  const float a0 = a[lane], a1 = a[lane + 32];
+  float v = a0 * __bfloat162float(b[lane]) + a1 * __bfloat162float(b[lane + 32]);
   v = warp_sum(v);
-  if (lane == 0) delta[w] = v;
+  const int l = m % Pc;
+  const size_t r = (static_cast<size_t>(m / Pc) * N + h) * Pc + l;
+  do16[r * kDh + lane] = __float2bfloat16_rn(a0);
+  do16[r * kDh + lane + 32] = __float2bfloat16_rn(a1);
+  if (lane == 0) {
+    delta[r] = v;
+    if (l % Lp >= L) lse[r] = INFINITY;
+  }
 }
 
-// head-major [M / Pc][N][Pc][64] fp32 <-> rows [M][N 64]: to_rows = 1 reads head-major x and
-// writes bf16 rows; to_rows = 0 reads fp32 rows and writes bf16 head-major
+// head-major [M / Pc][N][Pc][64] fp32 -> bf16 rows [M][N 64]
 __global__ void head_permute_kernel(const float* __restrict__ x, int M, int Pc, int N,
-                                    int to_rows, bf16* __restrict__ y) {
+                                    bf16* __restrict__ y) {
   const long long total = static_cast<long long>(M) * N * kDh;
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
     // i indexes the rows layout: row m, head h, element j
     const long long m = i / (static_cast<long long>(N) * kDh);
     const int h = static_cast<int>(i / kDh % N), j = static_cast<int>(i % kDh);
-    const long long hm = ((m / Pc * N + h) * Pc + m % Pc) * kDh + j;
-    if (to_rows) y[i] = __float2bfloat16_rn(x[hm]);
-    else y[hm] = __float2bfloat16_rn(x[i]);
+    y[i] = __float2bfloat16_rn(x[((m / Pc * N + h) * Pc + m % Pc) * kDh + j]);
   }
 }
 
@@ -567,8 +571,7 @@ struct fd_trainer_s {
     } band;
   } sB, sR;
   // scratch
-  bf16 *x0, *y16, *yh16, *a1, *vT, *kT, *do16, *dS, *P16, *dST, *PT, *QT, *dOT, *dy16, *dyT,
-      *xT, *dqkv16;
+  bf16 *x0, *y16, *yh16, *a1, *vT, *do16, *P16, *dy16, *dyT, *xT, *dqkv16;
   float *e, *z1, *F, *dF, *loss_part, *S, *delta, *dq2, *dk2, *dv1, *dqkv, *tq, *tk,
       *tv, *gA, *gB, *gC, *tbuf, *gtmp;
   int loss_blocks = 0;
@@ -699,11 +702,6 @@ struct Run {
     check(cudaMemcpyAsync(dst, src, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
     end();
   }
-  void zero(float* dst, size_t n) {
-    if (!begin(FD_TK_POINTWISE)) return;
-    check(cudaMemsetAsync(dst, 0, sizeof(float) * n, s));
-    end();
-  }
   void rmsnorm(const float* x, const float* g, int M, bf16* u) {
     if (!begin(FD_TK_NORM)) return;
     check(fd::launch_rmsnorm(x, g, M, tr->D, tr->eps, u, s));
@@ -799,7 +797,7 @@ void attn_fwd(Run& r, fd_trainer_s::Stack& st, int b) {
   }
   if (r.begin(FD_TK_POINTWISE)) {  // O rows (bf16) for the output projection
     const long long n = static_cast<long long>(M) * tr->NQ;
-    fd::train::head_permute_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(st.o32, M, Pc, N, 1,
+    fd::train::head_permute_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(st.o32, M, Pc, N,
                                                                          st.o[b]);
     r.check(cudaGetLastError());
     r.end();
@@ -807,60 +805,24 @@ void attn_fwd(Run& r, fd_trainer_s::Stack& st, int b) {
 }
 
 // attention backward of one block: dq2 (fp32, the head-major layout of q2), dk2, dv1 (fp32
-// [G][M][64], accumulated over the query chunks whose windows hold each key; the group's heads
-// sum inside each product) from dO (tr->gA, fp32 rows [M][N 64])
+// [G][M][64], summed over the query chunks whose windows hold each key and the group's heads)
+// from dO (tr->gA, fp32 rows [M][N 64])
 void attn_bwd(Run& r, fd_trainer_s::Stack& st, int b) {
   fd_trainer_s* tr = r.tr;
-  const int M = st.M, Pc = st.Pc, N = tr->N, hpg = N / tr->G, rows = tr->hs * Pc;
-  r.zero(tr->dk2, static_cast<size_t>(tr->G) * M * 64);
-  r.zero(tr->dv1, static_cast<size_t>(tr->G) * M * 64);
-  for (int g = 0; g < tr->G; ++g)
-    r.transpose(st.k2[b] + static_cast<size_t>(g) * M * 64, M, 64, 64,
-                tr->kT + static_cast<size_t>(g) * 64 * M, M);
-  // dO head-major (bf16) and delta = rowsum(dO o O) of every (chunk, head, row)
-  if (r.begin(FD_TK_POINTWISE)) {
-    const long long n = static_cast<long long>(M) * tr->NQ;
-    fd::train::head_permute_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(tr->gA, M, Pc, N, 0,
-                                                                         tr->do16);
-    r.check(cudaGetLastError());
-    r.end();
-  }
+  const int M = st.M, Pc = st.Pc, N = tr->N;
   if (r.begin(FD_TK_SOFTMAX)) {
-    const long long n = static_cast<long long>(M) * N * 32;
-    fd::train::delta_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(tr->gA, st.o[b], M, Pc, N,
-                                                                  tr->delta);
+    const long long threads = static_cast<long long>(M) * N * 32;
+    fd::train::attn_bwd_prep_kernel<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, r.s>>>(
+        tr->gA, st.o[b], M, Pc, tr->Lp, tr->L, N, tr->do16, tr->delta, st.lse[b]);
     r.check(cudaGetLastError());
     r.end();
   }
-  for (int i = 0; i < tr->T; ++i) {
-    const int j0 = i - tr->Wn + 1 > 0 ? i - tr->Wn + 1 : 0;
-    const int k0 = j0 * Pc, nk = (i + 1) * Pc - k0;
-    for (int h0 = 0; h0 < N; h0 += tr->hs) {
-      const int g = h0 / hpg;
-      const size_t q0 = (static_cast<size_t>(i) * N + h0) * Pc;
-      const bf16* Kw = st.k2[b] + (static_cast<size_t>(g) * M + k0) * 64;
-      const bf16* Vw = st.v1[b] + (static_cast<size_t>(g) * M + k0) * 64;
-      // S = Q K^T (recomputed) and dP = dO V^T in one launch, the softmax backward in its
-      // epilogue: dS = P (dP - delta) / sqrt(D_h) with P = exp(S / sqrt(D_h) - lse), written as
-      // dS, dS^T and P^T; S and dP are never stored
-      if (r.begin(FD_TK_ATTN_GEMM)) {
-        const fd::DsEpi ds{st.lse[b] + q0, tr->delta + q0, 0.125f, Pc, tr->Lp, tr->L,
-                           tr->dS, tr->dST, tr->PT};
-        r.check(fd::scores_bwd(rows, nk, st.q2[b] + q0 * 64, tr->do16 + q0 * 64, 64, Kw, Vw, 64,
-                               ds, tr->err, r.s));
-        r.end();
-      }
-      // dQ = dS K
-      r.gemm(FD_TK_ATTN_GEMM, fd::EPI_F32, rows, 64, nk, tr->dS, nk,
-             tr->kT + static_cast<size_t>(g) * 64 * M + k0, M, nullptr, tr->dq2 + q0 * 64, 64);
-      // dK += dS^T Q, dV += P^T dO (K of both products: the group's rows)
-      r.transpose(st.q2[b] + q0 * 64, rows, 64, 64, tr->QT, rows);
-      r.gemm(FD_TK_ATTN_GEMM, fd::EPI_RESID, nk, 64, rows, tr->dST, rows, tr->QT, rows, nullptr,
-             tr->dk2 + (static_cast<size_t>(g) * M + k0) * 64, 64);
-      r.transpose(tr->do16 + q0 * 64, rows, 64, 64, tr->dOT, rows);
-      r.gemm(FD_TK_ATTN_GEMM, fd::EPI_RESID, nk, 64, rows, tr->PT, rows, tr->dOT, rows, nullptr,
-             tr->dv1 + (static_cast<size_t>(g) * M + k0) * 64, 64);
-    }
+  if (r.begin(FD_TK_ATTN_GEMM)) {
+    const fd::AttnBwdParams p{st.lse[b], tr->delta, nullptr, nullptr, tr->T, N, tr->G, tr->Wn, Pc,
+                              tr->Lp, tr->L, M, tr->hs, tr->err};
+    r.check(fd::attention_bwd(st.q2[b], tr->do16, st.k2[b], st.v1[b], p, tr->dq2, tr->dk2, tr->dv1,
+                              r.s));
+    r.end();
   }
 }
 
@@ -1170,16 +1132,10 @@ fd_status fd_train_create(const fd_config* cfg, fd_weights w, int chunks, fd_tra
   tr->yh16 = dalloc<bf16>(tr, static_cast<size_t>(MR) * D, ok);
   tr->a1 = dalloc<bf16>(tr, static_cast<size_t>(MR) * D, ok);
   tr->vT = dalloc<bf16>(tr, static_cast<size_t>(G) * 64 * Mmax, ok);
-  tr->kT = dalloc<bf16>(tr, static_cast<size_t>(G) * 64 * Mmax, ok);
   tr->do16 = dalloc<bf16>(tr, static_cast<size_t>(Mmax) * NQ, ok);
-  tr->dS = dalloc<bf16>(tr, RK, ok);
   // S and P of the materialised forward (a stack whose band attention is off)
   const bool materialised = !tr->sB.band.on || !tr->sR.band.on;
   if (materialised) tr->P16 = dalloc<bf16>(tr, RK, ok);
-  tr->dST = dalloc<bf16>(tr, RK, ok);
-  tr->PT = dalloc<bf16>(tr, RK, ok);
-  tr->QT = dalloc<bf16>(tr, static_cast<size_t>(64) * tr->hs * Pmax, ok);
-  tr->dOT = dalloc<bf16>(tr, static_cast<size_t>(64) * tr->hs * Pmax, ok);
   tr->dy16 = dalloc<bf16>(tr, wide, ok);
   tr->dyT = dalloc<bf16>(tr, wide, ok);
   tr->xT = dalloc<bf16>(tr, wide, ok);

@@ -1295,6 +1295,20 @@ cudaError_t scores_bwd(int M, int N, const __nv_bfloat16* Q, const __nv_bfloat16
   return launch_gemm_scores_bwd(tq, tk, tdo, tv, p, num_sms(), s);
 }
 
+cudaError_t attention_bwd(const __nv_bfloat16* q, const __nv_bfloat16* dO, const __nv_bfloat16* k,
+                          const __nv_bfloat16* v, const AttnBwdParams& p, float* dq, float* dk,
+                          float* dv, cudaStream_t s) {
+  const uint64_t rows = static_cast<uint64_t>(p.T) * p.N * p.Pc;
+  const uint64_t keys = static_cast<uint64_t>(p.G) * p.M;
+  CUtensorMap tq, tdo, tk, tv;
+  if (!tmap_bf16(&tq, q, kHeadDim, rows, kHeadDim * 2, 64, 128) ||
+      !tmap_bf16(&tdo, dO, kHeadDim, rows, kHeadDim * 2, 64, 128) ||
+      !tmap_bf16(&tk, k, kHeadDim, keys, kHeadDim * 2, 64, 128) ||
+      !tmap_bf16(&tv, v, kHeadDim, keys, kHeadDim * 2, 64, 128))
+    return cudaErrorInvalidValue;
+  return launch_attention_bwd(tq, tdo, tk, tv, p, dq, dk, dv, s);
+}
+
 bool band_attention_maps(AttnStream* host, int T, int W, int rows_per_chunk, int G, int pitch,
                          const __nv_bfloat16* k, const __half* vt, const int* steps_dev,
                          int* err) {

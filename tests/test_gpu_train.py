@@ -248,3 +248,30 @@ def test_training_profile_counts_every_kind():
     assert torch.equal(grads, plain)
     tr.close()
     W.close()
+
+
+@pytest.mark.parametrize("lat_h,lat_w,chunks,window,r_t,heads,groups,qk", [
+    (2, 2, 2, 2, 1, 2, 2, False),     # one token per frame (127 padding keys), one head per group
+    (16, 16, 1, 1, 1, 2, 1, False),   # 64 tokens, a single chunk
+    (16, 32, 3, 2, 1, 4, 1, True),    # 128 tokens: no padding rows; all heads on one group
+    (6, 86, 3, 3, 2, 4, 2, False),    # 129 tokens: one token in the second tile; two refined frames
+    (30, 34, 2, 4, 4, 2, 2, False),   # 255 tokens, window longer than the clip, four frames
+])
+def test_attention_backward_tiles(lat_h, lat_w, chunks, window, r_t, heads, groups, qk):
+    """The step's fused attention backward at the edges of its 128-row query and key tiles, of
+    its windows and of its head groups, through every parameter's gradient (the bars above)."""
+    cfg = synth.FDConfig(latent_h=lat_h, latent_w=lat_w, patch=2, hidden=64 * heads, heads=heads,
+                         kv_groups=groups, n_blocks=1, n_refine=1 if r_t > 1 else 0,
+                         window=window, r_t=r_t, qk_norm=qk, chunks=chunks, name="tiles")
+    w, z = synth.make_weights(cfg), synth.make_latents(cfg)
+    x = synth.make_target_pixels(cfg, min_abs=0.3)
+    loss_ref, g_ref = training_step_explicit(cfg, w, z, x)
+    loss, flat = gpu_step(cfg, w, z, x)
+    assert abs(loss - loss_ref) <= LOSS_REL * abs(loss_ref)
+    for k, g in split(cfg, flat).items():
+        ref = g_ref[k].reshape(g.shape)
+        assert torch.isfinite(g).all(), k
+        # the gradients of Q and K rows vanish where a query sees one key (P = 1): held against
+        # the tensor's own scale plus fp32 noise of the whole step
+        err, scale = float((g - ref).norm()), float(ref.norm())
+        assert err <= GRAD_REL * scale + 1e-6, (k, err, scale)
