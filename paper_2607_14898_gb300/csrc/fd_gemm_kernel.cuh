@@ -158,7 +158,10 @@ __device__ __forceinline__ void rope_table(const QkvEpi& q, const float2* rope_t
 // in two TMEM accumulators; the epilogue turns them into dS = P (dP - delta) scale with P =
 // exp(S scale - lse) (p.ds), written as dS rows and dS^T, P^T columns (bf16). S and dP are never
 // stored.
-template <int BN, bool PAIR, int QKV, bool DS = false>
+// MN (the weight gradients, dW = dY^T X): A = dY^T and W = X^T with dY [K][M], X [K][N] row-major,
+// read as they are: a stage holds K rows of 64-column groups (3D boxes {64, 64 rows, groups}), MN-
+// major operands for the MMA, which the transposed copies of both matrices used to replace.
+template <int BN, bool PAIR, int QKV, bool DS = false, bool MN = false>
 __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmK,
@@ -197,6 +200,11 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
   const uint32_t full_tx = PAIR ? 2 * C::kStageBytes : C::kStageBytes;  // on rank 0's barrier
   const uint32_t bar_full0 = PAIR ? mapa_rank(bar_full, 0) : bar_full;
   auto load = [&](uint32_t dst, const CUtensorMap* m, int s, int x, int y) {
+    if (MN) {  // x = K row, y = first column
+      if (PAIR) tma_load_3d_pair(dst, m, bar_full0 + 8 * s, 0, x, y / 64);
+      else tma_load_3d(dst, m, bar_full + 8 * s, 0, x, y / 64);
+      return;
+    }
     if (PAIR) tma_load_2d_pair(dst, m, bar_full0 + 8 * s, x, y);
     else tma_load_2d(dst, m, bar_full + 8 * s, x, y);
   };
@@ -290,7 +298,8 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
     // ------------------------------------------------------------ MMA issuer
     // (the whole warp runs the loop; one elected lane issues)
     const uint32_t idesc =
-        p.fp8 ? idesc_e4m3_f32(tile_rows, BN) : idesc_bf16_f32(tile_rows, BN);
+        MN ? idesc_bf16_f32(tile_rows, BN) | (3u << 15)
+           : (p.fp8 ? idesc_e4m3_f32(tile_rows, BN) : idesc_bf16_f32(tile_rows, BN));
     int it = 0, tc = 0;
     bool ok = true;
     for (int tile = cta0; tile < tiles && ok; tile += ctas, ++tc) {
@@ -313,8 +322,12 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
         const uint32_t b0 = sB + s * C::kBBytes;
         // one 128-byte row of the stage: 4 MMAs of K = 16 bf16 (or 32 e4m3) elements
         static_assert(kBK == 64, "a K block is one 128-byte swizzle row of bf16");
-        const uint64_t da = sdesc_k_sw128(a0), db = sdesc_k_sw128(b0);
-        if (p.fp8) {
+        const uint64_t da = MN ? sdesc_mn_sw128(a0, kBK * 128) : sdesc_k_sw128(a0);
+        const uint64_t db = MN ? sdesc_mn_sw128(b0, kBK * 128) : sdesc_k_sw128(b0);
+        if (MN) {
+          if (PAIR) mma4_bf16_mn_pair_w(d_tmem, da, db, idesc, kb != 0);
+          else mma4_bf16_mn_w(d_tmem, da, db, idesc, kb != 0);
+        } else if (p.fp8) {
           if (PAIR) mma4_e4m3_ss_pair_w(d_tmem, da, db, idesc, kb != 0);
           else mma4_e4m3_ss_w(d_tmem, da, db, idesc, kb != 0);
         } else {
@@ -790,14 +803,14 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
   }
 }
 
-template <int BN, bool PAIR, int QKV, bool DS = false>
+template <int BN, bool PAIR, int QKV, bool DS = false, bool MN = false>
 static cudaError_t launch_bn(const CUtensorMap& tmA, const CUtensorMap& tmB,
                              const CUtensorMap& tmO, const CUtensorMap& tmK,
                              const CUtensorMap& tmV, const GemmParams& p, int num_sms,
                              cudaStream_t s) {
   using C = GemmCfg<BN, PAIR, QKV>;
   static const cudaError_t attr = cudaFuncSetAttribute(
-      gemm_kernel<BN, PAIR, QKV, DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
+      gemm_kernel<BN, PAIR, QKV, DS, MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
   if (attr != cudaSuccess) return attr;
   const int rows = PAIR ? 2 * kBM : kBM;
   const int tiles = ((p.M + rows - 1) / rows) * ((p.N + BN - 1) / BN);
@@ -820,7 +833,7 @@ static cudaError_t launch_bn(const CUtensorMap& tmA, const CUtensorMap& tmB,
     if (pairs == 0) {
       cfg.gridDim = dim3(2 * (num_sms / 2));
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<BN, PAIR, QKV>, &cfg) != cudaSuccess || n < 1) {
+      if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<BN, PAIR, QKV, DS, MN>, &cfg) != cudaSuccess || n < 1) {
         cudaGetLastError();
         n = num_sms / 2;
       }
@@ -830,7 +843,7 @@ static cudaError_t launch_bn(const CUtensorMap& tmA, const CUtensorMap& tmB,
   }
   const int units = tiles < slots ? tiles : slots;
   cfg.gridDim = dim3(PAIR ? 2 * units : units);
-  return cudaLaunchKernelEx(&cfg, gemm_kernel<BN, PAIR, QKV, DS>, tmA, tmB, tmO, tmK, tmV, p);
+  return cudaLaunchKernelEx(&cfg, gemm_kernel<BN, PAIR, QKV, DS, MN>, tmA, tmB, tmO, tmK, tmV, p);
 }
 
 template <int QKV>

@@ -206,6 +206,10 @@ cudaError_t launch_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const CU
 cudaError_t launch_gemm_scores_bwd(const CUtensorMap& tmA, const CUtensorMap& tmB,
                                    const CUtensorMap& tmdO, const CUtensorMap& tmV,
                                    const GemmParams& p, int num_sms, cudaStream_t s);
+// the weight-gradient instances (both operands MN-major), EPI_F32
+cudaError_t launch_gemm_wgrad(const CUtensorMap& tmA, const CUtensorMap& tmB,
+                              const CUtensorMap& tmO, const GemmParams& p, int bn, bool pair,
+                              int num_sms, cudaStream_t s);
 // the EPI_QKV instances (launch_gemm forwards to it for that epilogue)
 cudaError_t launch_gemm_qkv(const CUtensorMap& tmA, const CUtensorMap& tmB,
                             const CUtensorMap& tmO, const CUtensorMap& tmK,
@@ -283,6 +287,11 @@ void weights_add_user(fd_weights w, int delta);
 cudaError_t gemm_view(int epi, int M, int N, int K, const __nv_bfloat16* A, int lda,
                       const __nv_bfloat16* W, int ldw, const float* bias, float* out, int ldo,
                       int* err, cudaStream_t s);
+// dW[n_out][n_in] (fp32) = dY^T X with dY bf16 [rows][n_out] and X bf16 [rows][n_in] row-major;
+// n_out, n_in % 64 == 0, zero_bias: n_in zeros, 16-byte aligned pointers
+cudaError_t gemm_wgrad(int n_out, int n_in, int rows, const __nv_bfloat16* dY,
+                       const __nv_bfloat16* X, const float* zero_bias, float* dW, int* err,
+                       cudaStream_t s);
 // The attention's scores backward in one launch (the DS GEMM instance, 128 x 128 tiles):
 // S = Q K^T and dP = dO V^T (Q, dO bf16 [M][64] with row pitch ldq; K, V bf16 [N][64] with row
 // pitch ldk), then dS, dS^T, P^T as DsEpi describes. N % 32 == 0.

@@ -155,6 +155,24 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
       : "memory");
 }
 
+// 3D tile loads (x innermost), and the form that completes on an mbarrier of either CTA of a pair
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* m, uint32_t bar,
+                                            int x, int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* m,
+                                                 uint32_t bar_cluster, int x, int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      ".cta_group::2 [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
+
 // ---------------------------------------------------------------- CTA pairs (cta_group::2)
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
@@ -299,11 +317,11 @@ __device__ __forceinline__ void mma_commit_pair_w(uint32_t bar, uint16_t cta_mas
 // the peer's at the same offset), B's N rows split in halves the same way; each CTA's TMEM
 // receives its 128 rows of D.
 // Measured on the GB300 at 104-124 cycles per MMA against 125-126 for separate elected MMAs.
-#define FD_MMA4_BODY(KIND, GROUP)                                                          \
+#define FD_MMA4_BODY(KIND, GROUP, O1, O2, O3)                                              \
   "{\n\t.reg .pred p, q, e;\n\t.reg .b32 r;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"     \
   "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, %4, %4;\n\t"                                   \
-  "add.s64 a1, %1, 2;\n\tadd.s64 a2, %1, 4;\n\tadd.s64 a3, %1, 6;\n\t"                      \
-  "add.s64 b1, %2, 2;\n\tadd.s64 b2, %2, 4;\n\tadd.s64 b3, %2, 6;\n\t"                      \
+  "add.s64 a1, %1, " O1 ";\n\tadd.s64 a2, %1, " O2 ";\n\tadd.s64 a3, %1, " O3 ";\n\t"    \
+  "add.s64 b1, %2, " O1 ";\n\tadd.s64 b2, %2, " O2 ";\n\tadd.s64 b3, %2, " O3 ";\n\t"    \
   "elect.sync r|e, 0xffffffff;\n\t"                                                        \
   "@e tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], %1, %2, %3, p;\n\t"           \
   "@e tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], a1, b1, %3, q;\n\t"           \
@@ -311,28 +329,43 @@ __device__ __forceinline__ void mma_commit_pair_w(uint32_t bar, uint16_t cta_mas
   "@e tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], a3, b3, %3, q;\n\t}"
 __device__ __forceinline__ void mma4_bf16_ss_w(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                                uint32_t idesc, uint32_t accumulate) {
-  asm volatile(FD_MMA4_BODY("f16", "1") ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc),
+  asm volatile(FD_MMA4_BODY("f16", "1", "2", "4", "6") ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc),
                "r"(accumulate)
                : "memory");
 }
 __device__ __forceinline__ void mma4_e4m3_ss_w(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                                uint32_t idesc, uint32_t accumulate) {
-  asm volatile(FD_MMA4_BODY("f8f6f4", "1") ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc),
+  asm volatile(FD_MMA4_BODY("f8f6f4", "1", "2", "4", "6") ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc),
                "r"(accumulate)
                : "memory");
 }
 __device__ __forceinline__ void mma4_bf16_ss_pair_w(uint32_t d_tmem, uint64_t adesc,
                                                     uint64_t bdesc, uint32_t idesc,
                                                     uint32_t accumulate) {
-  asm volatile(FD_MMA4_BODY("f16", "2") ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc),
+  asm volatile(FD_MMA4_BODY("f16", "2", "2", "4", "6") ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc),
                "r"(accumulate)
                : "memory");
 }
 __device__ __forceinline__ void mma4_e4m3_ss_pair_w(uint32_t d_tmem, uint64_t adesc,
                                                     uint64_t bdesc, uint32_t idesc,
                                                     uint32_t accumulate) {
-  asm volatile(FD_MMA4_BODY("f8f6f4", "2") ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc),
+  asm volatile(FD_MMA4_BODY("f8f6f4", "2", "2", "4", "6") ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc),
                "r"(accumulate)
+               : "memory");
+}
+// Both operands MN-major (the instruction descriptor's transpose bits): K = 64 rows of 128 bytes,
+// 16 of them (2048 bytes, 128 in the encoded descriptor address) per MMA.
+__device__ __forceinline__ void mma4_bf16_mn_w(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+                                               uint32_t idesc, uint32_t accumulate) {
+  asm volatile(FD_MMA4_BODY("f16", "1", "128", "256", "384") ::"r"(d_tmem), "l"(adesc), "l"(bdesc),
+               "r"(idesc), "r"(accumulate)
+               : "memory");
+}
+__device__ __forceinline__ void mma4_bf16_mn_pair_w(uint32_t d_tmem, uint64_t adesc,
+                                                    uint64_t bdesc, uint32_t idesc,
+                                                    uint32_t accumulate) {
+  asm volatile(FD_MMA4_BODY("f16", "2", "128", "256", "384") ::"r"(d_tmem), "l"(adesc), "l"(bdesc),
+               "r"(idesc), "r"(accumulate)
                : "memory");
 }
 #undef FD_MMA4_BODY
@@ -510,6 +543,16 @@ __host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N) {
 // 128-byte swizzle. Advancing K by 16 elements inside an atom adds 32 B to the start.
 __device__ __forceinline__ uint64_t sdesc_k_sw128(uint32_t saddr) {
   return static_cast<uint64_t>((saddr >> 4) & 0x3FFFu) | (static_cast<uint64_t>(1) << 16) |
+         (static_cast<uint64_t>(1024 >> 4) << 32) | (static_cast<uint64_t>(1) << 46) |
+         (static_cast<uint64_t>(2) << 61);
+}
+
+// The same for an MN-major operand: K rows of 64 M (or N) elements (128 bytes, swizzled), 8-row
+// atoms 1024 B apart along K (the stride offset), groups of 64 M / N elements group_bytes apart
+// (the leading offset).
+__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t saddr, uint32_t group_bytes) {
+  return static_cast<uint64_t>((saddr >> 4) & 0x3FFFu) |
+         (static_cast<uint64_t>(group_bytes >> 4) << 16) |
          (static_cast<uint64_t>(1024 >> 4) << 32) | (static_cast<uint64_t>(1) << 46) |
          (static_cast<uint64_t>(2) << 61);
 }

@@ -571,9 +571,10 @@ struct fd_trainer_s {
     } band;
   } sB, sR;
   // scratch
-  bf16 *x0, *y16, *yh16, *a1, *vT, *do16, *P16, *dy16, *dyT, *xT, *dqkv16;
+  bf16 *x0, *y16, *yh16, *a1, *vT, *do16, *P16, *dy16, *dyT = nullptr, *xT = nullptr,
+      *dqkv16;
   float *e, *z1, *F, *dF, *loss_part, *S, *delta, *dq2, *dk2, *dv1, *dqkv, *tq, *tk,
-      *tv, *gA, *gB, *gC, *tbuf, *gtmp;
+      *tv, *gA, *gB, *gC, *tbuf, *gtmp = nullptr;
   int loss_blocks = 0;
   int hs = 1;  // heads of one KV group per attention product (a divisor of N / G)
   float* colsum_part = nullptr;  // partial column sums
@@ -718,8 +719,16 @@ struct Run {
     colsum(tr->tbuf, M, tr->D, tr->D, grad);
   }
   // weight gradient of a linear out = X W^T: dW [n_out][n_in] = dY^T X with dY16 [M][n_out]
-  // and X16 [M][n_in] (bf16; K of the product = M rows, padding rows of dY are zero)
+  // and X16 [M][n_in] (bf16; K of the product = M rows, padding rows of dY are zero), on the
+  // matrices as they are when both widths are whole 64-column groups
   void wgrad(const bf16* dY16, int n_out, const bf16* X16, int n_in, int M, float* dW) {
+    if (n_out % 64 == 0 && n_in % 64 == 0) {
+      if (!begin(FD_TK_WGRAD)) return;
+      check(fd::gemm_wgrad(n_out, n_in, M, dY16, X16, tr->zero_bias, dW, tr->err, s));
+      end();
+      return;
+    }
+    // narrow inputs (the patch embedding of a 48-channel latent)
     bf16* dyT = tr->dyT;
     bf16* xT = tr->xT;
     transpose(dY16, M, n_out, n_out, dyT, M);
@@ -1137,8 +1146,10 @@ fd_status fd_train_create(const fd_config* cfg, fd_weights w, int chunks, fd_tra
   const bool materialised = !tr->sB.band.on || !tr->sR.band.on;
   if (materialised) tr->P16 = dalloc<bf16>(tr, RK, ok);
   tr->dy16 = dalloc<bf16>(tr, wide, ok);
-  tr->dyT = dalloc<bf16>(tr, wide, ok);
-  tr->xT = dalloc<bf16>(tr, wide, ok);
+  if (tr->cin % 64) {
+    tr->dyT = dalloc<bf16>(tr, static_cast<size_t>(MB) * D, ok);
+    tr->xT = dalloc<bf16>(tr, static_cast<size_t>(MB) * tr->cin, ok);
+  }
   tr->dqkv16 = dalloc<bf16>(tr, wide, ok);
   tr->e = dalloc<float>(tr, static_cast<size_t>(MB) * tr->rt * D, ok);
   tr->z1 = dalloc<float>(tr, static_cast<size_t>(MR) * D, ok);
@@ -1166,8 +1177,7 @@ fd_status fd_train_create(const fd_config* cfg, fd_weights w, int chunks, fd_tra
   tr->gB = dalloc<float>(tr, wide, ok);
   tr->gC = dalloc<float>(tr, wide, ok);
   tr->tbuf = dalloc<float>(tr, static_cast<size_t>(Mmax) * D, ok);
-  tr->gtmp = dalloc<float>(tr, static_cast<size_t>(D) * std::max({D, tr->Dz, QO, tr->Cr, tr->cin}),
-                           ok);
+  if (tr->cin % 64) tr->gtmp = dalloc<float>(tr, static_cast<size_t>(D) * tr->cin, ok);
   if (tr->gated) {
     tr->dz32 = dalloc<float>(tr, static_cast<size_t>(Mmax) * tr->Dz, ok);
     tr->dwz = dalloc<float>(tr, static_cast<size_t>(tr->Dz) * (D + 1), ok);

@@ -1362,6 +1362,37 @@ cudaError_t gemm_view(int epi, int M, int N, int K, const __nv_bfloat16* A, int 
   return launch_gemm(ta, tb, to, to, to, p, t.bn, t.pair, num_sms(), s);
 }
 
+cudaError_t gemm_wgrad(int n_out, int n_in, int rows, const __nv_bfloat16* dY,
+                       const __nv_bfloat16* X, const float* zero_bias, float* dW, int* err,
+                       cudaStream_t s) {
+  if (n_out < 64 || n_in < 64 || rows < 1 || n_out % 64 || n_in % 64 || !aligned16(dY) ||
+      !aligned16(X) || !aligned16(dW) || !aligned16(zero_bias))
+    return cudaErrorInvalidValue;
+  const TileChoice t = pick_tile(n_out, n_in, rows, 64, false);
+  // [64 columns][rows][column groups] views; a stage's box: 64 rows of the tile's groups
+  auto map = [&](CUtensorMap* m, const __nv_bfloat16* x, int n, int tile_cols) {
+    const uint64_t dims[3] = {64, static_cast<uint64_t>(rows), static_cast<uint64_t>(n) / 64};
+    const uint64_t strides[2] = {static_cast<uint64_t>(n) * 2, 128};
+    const uint32_t box[3] = {64, kBK, static_cast<uint32_t>(tile_cols) / 64};
+    return tmap_nd(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, x, dims, strides, box,
+                   CU_TENSOR_MAP_SWIZZLE_128B);
+  };
+  CUtensorMap ta, tb, to;
+  if (!map(&ta, dY, n_out, 128) || !map(&tb, X, n_in, t.pair ? t.bn / 2 : t.bn) ||
+      !tmap_out_f32(&to, dW, n_in, n_out, n_in))
+    return cudaErrorInvalidValue;
+  GemmParams p{};
+  p.M = n_out;
+  p.N = n_in;
+  p.K = rows;
+  p.epi = EPI_F32;
+  p.bias = zero_bias;
+  p.out_f32 = dW;
+  p.ld_out = n_in;
+  p.err = err;
+  return launch_gemm_wgrad(ta, tb, to, p, t.bn, t.pair, num_sms(), s);
+}
+
 }  // namespace fd
 
 extern "C" {
