@@ -287,6 +287,10 @@ void weights_add_user(fd_weights w, int delta);
 cudaError_t gemm_view(int epi, int M, int N, int K, const __nv_bfloat16* A, int lda,
                       const __nv_bfloat16* W, int ldw, const float* bias, float* out, int ldo,
                       int* err, cudaStream_t s);
+// temporal upsampling of stacked chunks of Lp rows: y bf16 [M][D] times W [r_t D][D]^T + bias, column
+// block tau of row c Lp + l to row (c r_t + tau) Lp + l of out fp32 [M r_t][D]
+cudaError_t gemm_tup(int M, int rt, int Lp, int D, const __nv_bfloat16* y, const __nv_bfloat16* W,
+                     const float* bias, float* out, int* err, cudaStream_t s);
 // dW[n_out][n_in] (fp32) = dY^T X with dY bf16 [rows][n_out] and X bf16 [rows][n_in] row-major;
 // n_out, n_in % 64 == 0, zero_bias: n_in zeros, 16-byte aligned pointers
 cudaError_t gemm_wgrad(int n_out, int n_in, int rows, const __nv_bfloat16* dY,

@@ -28,35 +28,22 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <vector>
 
 #include "fd_internal.h"
+#include "fd_train_rows.cuh"
 #include "flashdec.h"
 
 namespace fd {
 namespace train {
 
-using bf16 = __nv_bfloat16;
-constexpr int kDh = kHeadDim;
-constexpr int kBandS = kHeadDim / 6;                  // pairs per spatial band (10)
-constexpr int kBandT = kHeadDim / 2 - 2 * kBandS;     // temporal pairs (12)
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
-}
-
-__global__ void to_bf16_kernel(const float* __restrict__ x, long long n, bf16* __restrict__ y) {
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x)
-    y[i] = __float2bfloat16_rn(x[i]);
 }
 
 // y[c][r] = x[r][c] for a rows x cols block (pitches in elements), through a padded tile
@@ -74,154 +61,6 @@ __global__ void transpose_kernel(const T* __restrict__ x, int rows, int cols, in
     const int c = c0 + i, r = r0 + threadIdx.x;
     if (r < rows && c < cols) y[static_cast<size_t>(c) * ldy + r] = tile[threadIdx.x][i];
   }
-}
-
-// GELU, exact (erf) form, and its derivative Phi(z) + z phi(z)
-__global__ void gelu_fwd_kernel(const float* __restrict__ z, long long n, bf16* __restrict__ a) {
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const float v = z[i];
-    a[i] = __float2bfloat16_rn(0.5f * v * (1.0f + erff(v * 0.70710678118654752f)));
-  }
-}
-__global__ void gelu_bwd_kernel(const float* __restrict__ z, const float* __restrict__ da,
-                                long long n, float* __restrict__ dz, bf16* __restrict__ dz16) {
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const float v = z[i];
-    const float Phi = 0.5f * (1.0f + erff(v * 0.70710678118654752f));
-    const float phi = 0.39894228040143268f * expf(-0.5f * v * v);
-    const float g = da[i] * (Phi + v * phi);
-    dz[i] = g;
-    dz16[i] = __float2bfloat16_rn(g);
-  }
-}
-
-// RMSNorm backward, one warp per row (y = x r g, r = (mean(x^2) + eps)^(-1/2), n = D):
-// dx = r (dy g) - x r^3 sum_j(dy_j g_j x_j) / n (+ add), t = dy x r (the gain's gradient
-// summed over rows)
-__global__ void rmsnorm_bwd_kernel(const float* __restrict__ x, const float* __restrict__ g,
-                                   const float* __restrict__ dy, const float* __restrict__ add,
-                                   int M, int D, float eps, float* __restrict__ dx,
-                                   float* __restrict__ t) {
-  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= M) return;
-  const float* xr = x + static_cast<size_t>(row) * D;
-  const float* dr = dy + static_cast<size_t>(row) * D;
-  float ss = 0.f, se = 0.f;
-  for (int j = lane; j < D; j += 32) {
-    const float v = xr[j];
-    ss = fmaf(v, v, ss);
-    se = fmaf(dr[j] * g[j], v, se);
-  }
-  ss = warp_sum(ss);
-  se = warp_sum(se);
-  const float r = rsqrtf(ss / D + eps);
-  const float c = r * r * r * se / D;
-  for (int j = lane; j < D; j += 32) {
-    const size_t k = static_cast<size_t>(row) * D + j;
-    float v = r * dr[j] * g[j] - xr[j] * c;
-    if (add != nullptr) v += add[k];
-    dx[k] = v;
-    t[k] = dr[j] * xr[j] * r;
-  }
-}
-
-// Gated MLP (the XL layout, reading R7): layer 1's output z [M][2 Dm] holds, on the device,
-// the gate and up columns of 32 hidden units side by side in blocks of 64 (gate unit 32 j + i
-// at column 64 j + i, its up column at 64 j + 32 + i); a = SiLU(gate) up, in unit order.
-__device__ __forceinline__ float logistic(float x) { return 1.0f / (1.0f + expf(-x)); }
-__global__ void swiglu_fwd_kernel(const float* __restrict__ z, long long M, int Dm,
-                                  bf16* __restrict__ a) {
-  const long long n = M * Dm;
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const long long m = i / Dm;
-    const int u = static_cast<int>(i % Dm);
-    const float* zr = z + m * 2 * Dm + (u / 32) * 64 + u % 32;
-    const float g = zr[0], up = zr[32];
-    a[i] = __float2bfloat16_rn(g * logistic(g) * up);
-  }
-}
-// its backward: d gate = da up SiLU'(gate) with SiLU'(x) = s(x) (1 + x (1 - s(x))), d up =
-// da SiLU(gate); dz in the interleaved layout, fp32 and a bf16 copy
-__global__ void swiglu_bwd_kernel(const float* __restrict__ z, const float* __restrict__ da,
-                                  long long M, int Dm, float* __restrict__ dz,
-                                  bf16* __restrict__ dz16) {
-  const long long n = M * Dm;
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const long long m = i / Dm;
-    const int u = static_cast<int>(i % Dm);
-    const long long c = m * 2 * Dm + (u / 32) * 64 + u % 32;
-    const float g = z[c], up = z[c + 32], d = da[i];
-    const float sg = logistic(g);
-    const float dg = d * up * sg * (1.0f + g * (1.0f - sg)), du = d * g * sg;
-    dz[c] = dg;
-    dz[c + 32] = du;
-    dz16[c] = __float2bfloat16_rn(dg);
-    dz16[c + 32] = __float2bfloat16_rn(du);
-  }
-}
-// rows of a gated layer 1's gradient from the device's interleaved order back to the blob's
-// (gate rows, then up rows): dst row r = src row of blob row r
-__global__ void gated_rows_kernel(const float* __restrict__ src, int rows, int len,
-                                  float* __restrict__ dst) {
-  const long long n = static_cast<long long>(rows) * len;
-  const int gate = rows / 2;
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int r = static_cast<int>(i / len), k = static_cast<int>(i % len);
-    const int u = r < gate ? r : r - gate;
-    const int dr = (u / 32) * 64 + (r < gate ? 0 : 32) + u % 32;
-    dst[i] = src[static_cast<size_t>(dr) * len + k];
-  }
-}
-
-// out[c] = sum over rows of x[r][c], rows in order (deterministic)
-__global__ void colsum_kernel(const float* __restrict__ x, long long rows, int cols, int ld,
-                              float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (long long r = 0; r < rows; ++r) s += x[r * ld + c];
-  out[c] = s;
-}
-
-// The same sums in two stages, for many rows: part[k][c] = the sum of rows k R .. k R + R - 1
-// (in order), then out[c] = the sum of the parts in order. A fixed order, so repeatable bits.
-constexpr int kColsumRows = 256;
-__global__ void colsum_part_kernel(const float* __restrict__ x, long long rows, int cols, int ld,
-                                   float* __restrict__ part) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  const long long r0 = static_cast<long long>(blockIdx.y) * kColsumRows;
-  const long long r1 = r0 + kColsumRows < rows ? r0 + kColsumRows : rows;
-  float s = 0.f;
-  for (long long r = r0; r < r1; ++r) s += x[r * ld + c];
-  part[static_cast<size_t>(blockIdx.y) * cols + c] = s;
-}
-__global__ void colsum_finish_kernel(const float* __restrict__ part, int parts, int cols,
-                                     float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int k = 0; k < parts; ++k) s += part[static_cast<size_t>(k) * cols + c];
-  out[c] = s;
-}
-
-// RoPE tables (host-computed in double): temporal (cos, sin) [frames][kBandT], row and column
-// [grid][kBandS]
-struct Rope {
-  const float2 *t, *y, *x;
-};
-
-// angle of pair i for frame f, grid row gy, column gx
-__device__ __forceinline__ float2 rope_cs(const Rope& rp, int i, int f, int gy, int gx) {
-  if (i < kBandT) return rp.t[f * kBandT + i];
-  if (i < kBandT + kBandS) return rp.y[gy * kBandS + i - kBandT];
-  return rp.x[gx * kBandS + i - kBandT - kBandS];
 }
 
 // RMS over the 64 values of one head with gain g
@@ -293,74 +132,6 @@ __global__ void qkv_fwd_kernel(const float* __restrict__ qkv, int M, int Pc, int
 #pragma unroll
     for (int j = 0; j < kDh; ++j) d[static_cast<size_t>(j) * pitch] = __float2half_rn(v[j]);
   }
-}
-
-// RMS over one head, backward: x the pre-norm values, dy the gradient of the normed output
-// (overwritten by dx); t = dy x r (gain's gradient term)
-__device__ __forceinline__ void head_rms_bwd(const float (&x)[kDh], float (&dy)[kDh],
-                                             const float* g, float eps, float* t) {
-  float ss = 0.f, se = 0.f;
-#pragma unroll
-  for (int j = 0; j < kDh; ++j) {
-    ss = fmaf(x[j], x[j], ss);
-    se = fmaf(dy[j] * g[j], x[j], se);
-  }
-  const float r = rsqrtf(ss / kDh + eps);
-  const float c = r * r * r * se / kDh;
-#pragma unroll
-  for (int j = 0; j < kDh; ++j) {
-    t[j] = dy[j] * x[j] * r;
-    dy[j] = r * dy[j] * g[j] - x[j] * c;
-  }
-}
-
-// QKV backward of every row: dq2 fp32 [M / Pc][N][Pc][64] (the layout of q2), dk2 / dv1 fp32
-// [G][M][64] -> dqkv fp32
-// [M][(N + 2G) 64] (inverse RoPE: the rotation by the negated angle; then the per-head RMS
-// backward where the forward normalised); gain terms tq [M N][64] (qk_norm), tk / tv [M G][64]
-__global__ void qkv_bwd_kernel(const float* __restrict__ qkv, const float* __restrict__ dq2,
-                               const float* __restrict__ dk2, const float* __restrict__ dv1,
-                               int M, int Pc, int Lp, int L, int gw, int N, int G, int qk_norm,
-                               const float* __restrict__ gk, const float* __restrict__ g2,
-                               float eps, Rope rp, float* __restrict__ dqkv,
-                               float* __restrict__ tq, float* __restrict__ tk,
-                               float* __restrict__ tv) {
-  const int slots = N + 2 * G;
-  const long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-  if (idx >= static_cast<long long>(M) * slots) return;
-  const int row = static_cast<int>(idx / slots), slot = static_cast<int>(idx % slots);
-  const int f = row / Lp, l = min(row % Lp, L - 1);  // padding rows take a real token's angles
-  const int gy = l / gw, gx = l % gw;
-  const bool is_q = slot < N, is_k = !is_q && slot < N + G;
-  float d[kDh], x[kDh];
-  const float* src;
-  if (is_q) src = dq2 + (static_cast<size_t>(row / Pc * N + slot) * Pc + row % Pc) * kDh;
-  else if (is_k) src = dk2 + (static_cast<size_t>(slot - N) * M + row) * kDh;
-  else src = dv1 + (static_cast<size_t>(slot - N - G) * M + row) * kDh;
-#pragma unroll
-  for (int j = 0; j < kDh; ++j) d[j] = src[j];
-  if (is_q || is_k) {
-#pragma unroll
-    for (int i = 0; i < kDh / 2; ++i) {
-      const float2 cs = rope_cs(rp, i, f, gy, gx);
-      const float a = d[2 * i], b = d[2 * i + 1];
-      d[2 * i] = a * cs.x + b * cs.y;
-      d[2 * i + 1] = -a * cs.y + b * cs.x;
-    }
-  }
-  const float* pre = qkv + static_cast<size_t>(row) * slots * kDh + slot * kDh;
-#pragma unroll
-  for (int j = 0; j < kDh; ++j) x[j] = pre[j];
-  if (is_k) {
-    head_rms_bwd(x, d, gk, eps, tk + (static_cast<size_t>(row) * G + slot - N) * kDh);
-  } else if (is_q && qk_norm) {
-    head_rms_bwd(x, d, g2, eps, tq + (static_cast<size_t>(row) * N + slot) * kDh);
-  } else if (!is_q && !qk_norm) {
-    head_rms_bwd(x, d, g2, eps, tv + (static_cast<size_t>(row) * G + slot - N - G) * kDh);
-  }
-  float* dst = dqkv + static_cast<size_t>(row) * slots * kDh + slot * kDh;
-#pragma unroll
-  for (int j = 0; j < kDh; ++j) dst[j] = d[j];
 }
 
 // Band softmax of one (query chunk, KV group): S fp32 [rows][n] (row pitch n), rows = the
@@ -435,90 +206,6 @@ __global__ void head_permute_kernel(const float* __restrict__ x, int M, int Pc, 
   }
 }
 
-// L1 term of the pixels (reading T3: the mean of |x_hat - x| over the clip, unclamped output,
-// reading T1) through the pixel shuffle: F [R][C rs^2] with refined row (c r_t + tau) Lp + l,
-// target [T][C][r_t][H][W]; dF = sign(F - x) / total (0 on padding rows, and on chunk 0's
-// frames tau >= first, which a one-frame first chunk does not emit); per-block partial sums of
-// |F - x| into part[blockIdx.x] (fixed-order tree)
-__global__ void l1_head_kernel(const float* __restrict__ F, const float* __restrict__ target,
-                               int T, int rt, int first, int Lp, int L, int gh, int gw, int C,
-                               int rs, float inv_total, float* __restrict__ dF,
-                               float* __restrict__ part) {
-  __shared__ float red[256];
-  const int cols = C * rs * rs;
-  const long long total = static_cast<long long>(T) * rt * Lp * cols;
-  const long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-  float e = 0.f;
-  if (i < total) {
-    const long long row = i / cols;
-    const int col = static_cast<int>(i % cols);
-    const int l = static_cast<int>(row % Lp);
-    const long long ft = row / Lp;  // c r_t + tau
-    float g = 0.f;
-    const int c = static_cast<int>(ft / rt), tau = static_cast<int>(ft % rt);
-    if (l < L && (c > 0 || tau < first)) {
-      const int ch = col / (rs * rs), ij = col % (rs * rs);
-      const int ii = ij / rs, jj = ij % rs;
-      const int h = l / gw, w = l % gw;
-      const int H = gh * rs, W = gw * rs;
-      const float x = target[((static_cast<size_t>(c) * C + ch) * rt + tau) * H * W +
-                             static_cast<size_t>(h * rs + ii) * W + w * rs + jj];
-      const float diff = F[i] - x;
-      e = fabsf(diff);
-      g = diff > 0.f ? inv_total : (diff < 0.f ? -inv_total : 0.f);
-    }
-    dF[i] = g;
-  }
-  red[threadIdx.x] = e;
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-
-// one block of kLossThreads: thread t sums parts t, t + kLossThreads, ... in fp64, then a
-// fixed-order tree over the threads (the same bits every step)
-constexpr int kLossThreads = 1024;
-__global__ void finish_loss_kernel(const float* __restrict__ part, int n, float inv_total,
-                                   float* __restrict__ loss) {
-  __shared__ double acc[kLossThreads];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += kLossThreads) s += part[i];
-  acc[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = kLossThreads / 2; w > 0; w >>= 1) {
-    if (static_cast<int>(threadIdx.x) < w) acc[threadIdx.x] += acc[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *loss = static_cast<float>(acc[0] * inv_total);
-}
-
-// temporal upsampling layout (Eq. temporal_upsample, reading R6): channel block tau of token
-// row c Lp + l of e [T Lp][r_t D] is refined row (c r_t + tau) Lp + l of hf [T r_t Lp][D]
-__global__ void tup_permute_kernel(const float* __restrict__ src, int T, int rt, int Lp, int D,
-                                   int inverse, float* __restrict__ dst, bf16* __restrict__ dst16) {
-  const long long total = static_cast<long long>(T) * rt * Lp * D;
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    // i indexes e: row c Lp + l, column tau D + d
-    const long long erow = i / (static_cast<long long>(rt) * D);
-    const int ecol = static_cast<int>(i % (static_cast<long long>(rt) * D));
-    const int c = static_cast<int>(erow / Lp), l = static_cast<int>(erow % Lp);
-    const int tau = ecol / D, d = ecol % D;
-    const long long hrow = (static_cast<long long>(c) * rt + tau) * Lp + l;
-    const long long h = hrow * D + d;
-    if (inverse) {
-      const float v = src[h];
-      dst[i] = v;
-      dst16[i] = __float2bfloat16_rn(v);
-    } else {
-      dst[h] = src[i];
-    }
-  }
-}
-
 }  // namespace train
 }  // namespace fd
 
@@ -534,7 +221,7 @@ struct fd_trainer_s {
   int Dz = 0;          // MLP layer 1's outputs: Dm, or 2 Dm for the gated MLP (interleaved)
   bool gated = false;  // gated-SiLU MLP (the XL layout)
   bool f1 = false;     // chunk 0 emits one frame (first_chunk_frames = 1)
-  float *dz32 = nullptr, *dwz = nullptr;  // gated: dz [M][2 Dm], layer 1's gradients (device order)
+  float* dwz = nullptr;  // gated: layer 1's weight gradient (device order)
   float eps;
   std::vector<const void*> wt;   // device tensors of the weights, blob order
   std::vector<size_t> goff;      // element offset of each tensor in the gradient blob
@@ -573,12 +260,10 @@ struct fd_trainer_s {
   // scratch
   bf16 *x0, *y16, *yh16, *a1, *vT, *do16, *P16, *dy16, *dyT = nullptr, *xT = nullptr,
       *dqkv16;
-  float *e, *z1, *F, *dF, *loss_part, *S, *delta, *dq2, *dk2, *dv1, *dqkv, *tq, *tk,
-      *tv, *gA, *gB, *gC, *tbuf, *gtmp = nullptr;
-  int loss_blocks = 0;
+  float *z1, *F, *loss_part, *S, *delta, *dq2, *dk2, *dv1, *gA, *gB, *gC, *gtmp = nullptr;
   int hs = 1;  // heads of one KV group per attention product (a divisor of N / G)
-  float* colsum_part = nullptr;  // partial column sums
-  size_t colsum_elems = 0;
+  float *part_a = nullptr, *part_b = nullptr;  // partial column sums, two sets of part_elems
+  size_t part_elems = 0;
   // per-kernel profile (fd_train_profile_enable): events around each launch, by kernel kind
   struct Rec {
     int kind;
@@ -629,6 +314,14 @@ double rope_inv_freq(int i, double base) {
   return std::pow(base, -2.0 * j / d);
 }
 
+constexpr int kQkvBwdSmem = 2 * fd::train::kQkvUnits * fd::train::kQkvPad * 4;
+
+// thread groups that share a block's rows in the RMSNorm backward (one for D >= 1024)
+int norm_groups(int D) {
+  const int threads = (D + 3) / 4;
+  return threads >= 256 ? 1 : std::min(fd::train::kNormRows, 256 / threads);
+}
+
 // the launches of one step, in order on one stream; any failure ends the step
 struct Run {
   fd_trainer_s* tr;
@@ -668,12 +361,6 @@ struct Run {
                         tr->err, s));
     end();
   }
-  void bf(const float* x, long long n, bf16* y) {
-    if (!begin(FD_TK_POINTWISE)) return;
-    fd::train::to_bf16_kernel<<<blocks_for(n, 256), 256, 0, s>>>(x, n, y);
-    check(cudaGetLastError());
-    end();
-  }
   template <typename T>
   void transpose(const T* x, int rows, int cols, int ldx, T* y, int ldy) {
     if (!begin(FD_TK_TRANSPOSE)) return;
@@ -682,21 +369,24 @@ struct Run {
     check(cudaGetLastError());
     end();
   }
-  void colsum(const float* x, long long rows, int cols, int ld, float* out) {
-    const int parts = static_cast<int>((rows + fd::train::kColsumRows - 1) /
-                                       fd::train::kColsumRows);
-    if (static_cast<size_t>(parts) * cols > tr->colsum_elems) {
-      ok = false;
-      return;
+  // room for `parts` partial rows of `cols` columns
+  bool room(size_t parts, size_t cols) {
+    if (parts * cols > tr->part_elems) ok = false;
+    return ok;
+  }
+  // the last step of up to three column sums, in the same launch bracket as their partial sums
+  void sum_parts(std::initializer_list<fd::train::SumJob> jobs) {
+    fd::train::SumJobs js{};
+    int n = 0, cols = 0;
+    for (const fd::train::SumJob& j : jobs) {
+      if (j.out == nullptr) continue;
+      js.job[n++] = j;
+      cols = std::max(cols, j.cols);
     }
-    if (!begin(FD_TK_POINTWISE)) return;
-    fd::train::colsum_part_kernel<<<dim3((cols + 127) / 128, parts), 128, 0, s>>>(
-        x, rows, cols, ld, tr->colsum_part);
+    if (n == 0) return;
+    fd::train::sum_parts_kernel<<<dim3((cols + 31) / 32, n), dim3(32, fd::train::kSumRows), 0, s>>>(
+        js);
     check(cudaGetLastError());
-    fd::train::colsum_finish_kernel<<<(cols + 127) / 128, 128, 0, s>>>(tr->colsum_part, parts,
-                                                                      cols, out);
-    check(cudaGetLastError());
-    end();
   }
   void copy(float* dst, const float* src, size_t n) {
     if (!begin(FD_TK_POINTWISE)) return;
@@ -708,15 +398,30 @@ struct Run {
     check(fd::launch_rmsnorm(x, g, M, tr->D, tr->eps, u, s));
     end();
   }
-  // dx = RMSNorm backward (+ add), the gain's gradient into grad
+  // dx = RMSNorm backward (+ add) in fp32 and bf16, the gain's gradient into grad, the column sums
+  // of dx (the bias gradient of the linear whose output gradient dx is) into bias_grad if non-null
   void rmsnorm_bwd(const float* x, const float* g, const float* dy, const float* add, int M,
-                   float* dx, float* grad) {
-    if (!begin(FD_TK_NORM)) return;
-    fd::train::rmsnorm_bwd_kernel<<<(M + 7) / 8, 256, 0, s>>>(x, g, dy, add, M, tr->D, tr->eps,
-                                                             dx, tr->tbuf);
+                   float* dx, bf16* dx16, float* grad, float* bias_grad) {
+    using namespace fd::train;
+    const int D = tr->D, groups = norm_groups(D);
+    const int blocks = (M + kNormRows - 1) / kNormRows, parts = blocks * groups;
+    if (!room(parts, D) || !begin(FD_TK_NORM)) return;
+    rmsnorm_bwd_kernel<4><<<blocks, 256, 0, s>>>(x, g, dy, add, M, D, tr->eps, groups, dx, dx16,
+                                                tr->part_a, bias_grad ? tr->part_b : nullptr);
     check(cudaGetLastError());
+    sum_parts({{tr->part_a, parts, D, D, 0, grad}, {tr->part_b, parts, D, D, 0, bias_grad}});
     end();
-    colsum(tr->tbuf, M, tr->D, tr->D, grad);
+  }
+  // dz16 = da GELU'(z) (bf16) and the bias gradient, its column sums; cols % 4 == 0
+  void gelu_bwd(const float* z, const float* da, int M, int cols, bf16* dz16, float* bias_grad) {
+    using namespace fd::train;
+    const int parts = (M + kRowBlock - 1) / kRowBlock;
+    if (!room(parts, cols) || !begin(FD_TK_POINTWISE)) return;
+    gelu_bwd_sum_kernel<<<dim3((cols + 1023) / 1024, parts), 256, 0, s>>>(z, da, M, cols, dz16,
+                                                                         tr->part_a);
+    check(cudaGetLastError());
+    sum_parts({{tr->part_a, parts, cols, cols, 0, bias_grad}});
+    end();
   }
   // weight gradient of a linear out = X W^T: dW [n_out][n_in] = dY^T X with dY16 [M][n_out]
   // and X16 [M][n_in] (bf16; K of the product = M rows, padding rows of dY are zero), on the
@@ -862,10 +567,11 @@ void block_fwd(Run& r, fd_trainer_s::Stack& st, int b, size_t e0) {
   if (r.begin(FD_TK_POINTWISE)) {
     const long long n = static_cast<long long>(M) * tr->Dm;
     if (tr->gated)
-      fd::train::swiglu_fwd_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(st.z[b], M, tr->Dm,
-                                                                         st.a[b]);
+      fd::train::swiglu_fwd_kernel<<<blocks_for(n / 4, 256), 256, 0, r.s>>>(st.z[b], M, tr->Dm,
+                                                                             st.a[b]);
     else
-      fd::train::gelu_fwd_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(st.z[b], n, st.a[b]);
+      fd::train::gelu_fwd_kernel<<<blocks_for(n / 4, 256), 256, 0, r.s>>>(
+          reinterpret_cast<const float4*>(st.z[b]), n / 4, reinterpret_cast<uint2*>(st.a[b]));
     r.check(cudaGetLastError());
     r.end();
   }
@@ -874,85 +580,76 @@ void block_fwd(Run& r, fd_trainer_s::Stack& st, int b, size_t e0) {
          r.wf(e0 + kM2B), st.h[b + 1], tr->D);
 }
 
-// one block backward: dho (tr->gB, fp32 [M][D]) -> dh_in (tr->gB), gradients into g
+// one block backward: dho (tr->gB, fp32 [M][D], and its bf16 copy tr->dy16; the gradient of this
+// block's second MLP bias is its column sums, already taken) -> dh_in (tr->gB and tr->dy16),
+// gradients into g; prev_bias: where the column sums of dh_in belong (the bias gradient of what
+// produced the block's input), or null
 void block_bwd(Run& r, fd_trainer_s::Stack& st, int b, size_t e0,
-               const fd_trainer_s::LinT& lt, float* g) {
+               const fd_trainer_s::LinT& lt, float* g, float* prev_bias) {
   fd_trainer_s* tr = r.tr;
   const int M = st.M, D = tr->D, Dm = tr->Dm, NQ = tr->NQ, QO = tr->QO;
-  float* dho = tr->gB;
-  r.bf(dho, static_cast<long long>(M) * D, tr->dy16);
   // MLP layer 2
   r.gemm(FD_TK_DGRAD, fd::EPI_F32, M, Dm, D, tr->dy16, D, lt.mlp2, D, nullptr, tr->gC, Dm);  // da
   r.wgrad(tr->dy16, D, st.a[b], Dm, M, r.grad(g, e0 + kM2W));
-  r.colsum(dho, M, D, D, r.grad(g, e0 + kM2B));
   // GELU' (or the gated SiLU's derivative into the interleaved dz)
   const int Dz = tr->Dz;
-  float* dz = tr->gated ? tr->dz32 : tr->gC;
-  if (r.begin(FD_TK_POINTWISE)) {
-    const long long n = static_cast<long long>(M) * Dm;
-    if (tr->gated)
-      fd::train::swiglu_bwd_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(st.z[b], tr->gC, M, Dm,
-                                                                          dz, tr->dqkv16);
-    else
-      fd::train::gelu_bwd_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(st.z[b], tr->gC, n,
-                                                                        tr->gC, tr->dqkv16);
-    r.check(cudaGetLastError());
-    r.end();
+  if (tr->gated) {
+    const int parts = (M + fd::train::kRowBlock - 1) / fd::train::kRowBlock;
+    if (r.room(parts, Dz) && r.begin(FD_TK_POINTWISE)) {
+      fd::train::swiglu_bwd_sum_kernel<<<dim3((Dm + 1023) / 1024, parts), 256, 0, r.s>>>(
+          st.z[b], tr->gC, M, Dm, tr->dqkv16, tr->part_a);
+      r.check(cudaGetLastError());
+      r.sum_parts({{tr->part_a, parts, Dz, Dz, Dm, r.grad(g, e0 + kM1B)}});
+      r.end();
+    }
+  } else {
+    r.gelu_bwd(st.z[b], tr->gC, M, Dm, tr->dqkv16, r.grad(g, e0 + kM1B));
   }
   // MLP layer 1
   r.gemm(FD_TK_DGRAD, fd::EPI_F32, M, D, Dz, tr->dqkv16, Dz, lt.mlp1, Dz, nullptr, tr->gA, D);  // du2
-  if (tr->gated) {  // gradients in the device's interleaved rows, then into the blob's order
-    float* dwz = tr->dwz;
-    float* dbz = tr->dwz + static_cast<size_t>(Dz) * D;
-    r.wgrad(tr->dqkv16, Dz, st.u2[b], D, M, dwz);
-    r.colsum(dz, M, Dz, Dz, dbz);
+  if (tr->gated) {  // the weight gradient in the device's interleaved rows, then in the blob's order
+    r.wgrad(tr->dqkv16, Dz, st.u2[b], D, M, tr->dwz);
     if (r.begin(FD_TK_POINTWISE)) {
-      const long long n = static_cast<long long>(Dz) * D;
+      const long long n = static_cast<long long>(Dz) * D / 4;
       fd::train::gated_rows_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(
-          dwz, Dz, D, r.grad(g, e0 + kM1W));
-      r.check(cudaGetLastError());
-      fd::train::gated_rows_kernel<<<blocks_for(Dz, 256), 256, 0, r.s>>>(
-          dbz, Dz, 1, r.grad(g, e0 + kM1B));
+          reinterpret_cast<const float4*>(tr->dwz), Dz, D / 4,
+          reinterpret_cast<float4*>(r.grad(g, e0 + kM1W)));
       r.check(cudaGetLastError());
       r.end();
     }
   } else {
     r.wgrad(tr->dqkv16, Dz, st.u2[b], D, M, r.grad(g, e0 + kM1W));
-    r.colsum(dz, M, Dz, Dz, r.grad(g, e0 + kM1B));
   }
-  // RMSNorm 2, plus the residual
-  r.rmsnorm_bwd(st.hm[b], r.wf(e0 + kN2), tr->gA, dho, M, tr->gC, r.grad(g, e0 + kN2));
-  float* dhm = tr->gC;
-  r.bf(dhm, static_cast<long long>(M) * D, tr->dy16);
+  // RMSNorm 2, plus the residual: dhm (gC, dy16); its column sums are the output bias's gradient
+  r.rmsnorm_bwd(st.hm[b], r.wf(e0 + kN2), tr->gA, tr->gB, M, tr->gC, tr->dy16,
+                r.grad(g, e0 + kN2), r.grad(g, e0 + kOB));
   // output projection
   r.gemm(FD_TK_DGRAD, fd::EPI_F32, M, NQ, D, tr->dy16, D, lt.out, D, nullptr, tr->gA, NQ);  // dO (fp32)
   r.wgrad(tr->dy16, D, st.o[b], NQ, M, r.grad(g, e0 + kOW));
-  r.colsum(dhm, M, D, D, r.grad(g, e0 + kOB));
   // attention (reads dO from gA)
   attn_bwd(r, st, b);
-  // KV-norm / QK-norm and RoPE backward
-  if (r.begin(FD_TK_NORM)) {
+  // KV-norm / QK-norm and RoPE backward, the bias's and the two gains' gradients
+  const int slots = tr->N + 2 * tr->G;
+  const int bx = M / fd::train::kQkvRows;
+  const int by = (slots + fd::train::kQkvSlots - 1) / fd::train::kQkvSlots;
+  if (r.room(bx, QO) && r.room(static_cast<size_t>(bx) * by, 128) && r.begin(FD_TK_NORM)) {
     const fd::train::Rope rp{tr->rope_t, tr->rope_y, tr->rope_x};
-    const long long n = static_cast<long long>(M) * (tr->N + 2 * tr->G);
-    fd::train::qkv_bwd_kernel<<<blocks_for(n, 128), 128, 0, r.s>>>(
-        st.qkv[b], tr->dq2, tr->dk2, tr->dv1, M, st.Pc, tr->Lp, tr->L, tr->gw, tr->N, tr->G,
-        tr->cfg.qk_norm, r.wf(e0 + kKG), r.wf(e0 + kG2), tr->eps, rp, tr->dqkv, tr->tq, tr->tk,
-        tr->tv);
+    const fd::train::QkvShape sh{M, st.Pc, tr->Lp, tr->L, tr->gw, tr->N, tr->G, tr->cfg.qk_norm};
+    fd::train::qkv_bwd_kernel<<<dim3(bx, by), fd::train::kQkvUnits, kQkvBwdSmem, r.s>>>(
+        st.qkv[b], tr->dq2, tr->dk2, tr->dv1, sh, r.wf(e0 + kKG), r.wf(e0 + kG2), tr->eps, rp,
+        tr->dqkv16, tr->part_a, tr->part_b);
     r.check(cudaGetLastError());
+    r.sum_parts({{tr->part_a, bx, QO, QO, 0, r.grad(g, e0 + kQB)},
+                 {tr->part_b, bx * by, 128, 64, 0, r.grad(g, e0 + kKG)},
+                 {tr->part_b + 64, bx * by, 128, 64, 0, r.grad(g, e0 + kG2)}});
     r.end();
   }
-  r.colsum(tr->tk, static_cast<long long>(M) * tr->G, 64, 64, r.grad(g, e0 + kKG));
-  if (tr->cfg.qk_norm)
-    r.colsum(tr->tq, static_cast<long long>(M) * tr->N, 64, 64, r.grad(g, e0 + kG2));
-  else
-    r.colsum(tr->tv, static_cast<long long>(M) * tr->G, 64, 64, r.grad(g, e0 + kG2));
-  r.bf(tr->dqkv, static_cast<long long>(M) * QO, tr->dqkv16);
   // QKV projection
   r.gemm(FD_TK_DGRAD, fd::EPI_F32, M, D, QO, tr->dqkv16, QO, lt.qkv, QO, nullptr, tr->gA, D);  // du
   r.wgrad(tr->dqkv16, QO, st.u[b], D, M, r.grad(g, e0 + kQW));
-  r.colsum(tr->dqkv, M, QO, QO, r.grad(g, e0 + kQB));
   // RMSNorm 1, plus the residual: dh_in
-  r.rmsnorm_bwd(st.h[b], r.wf(e0 + kN1), tr->gA, dhm, M, tr->gB, r.grad(g, e0 + kN1));
+  r.rmsnorm_bwd(st.h[b], r.wf(e0 + kN1), tr->gA, tr->gC, M, tr->gB, tr->dy16,
+                r.grad(g, e0 + kN1), prev_bias);
 }
 
 }  // namespace
@@ -970,6 +667,9 @@ fd_status fd_train_create(const fd_config* cfg, fd_weights w, int chunks, fd_tra
   // the bf16-valued decoder: GELU or gated-SiLU MLPs, r_t frames per chunk or one from chunk 0
   if (cfg->mlp_fp8) return FD_ERR_CONFIG;
   if (chunks < 1 || chunks > 256) return FD_ERR_INVALID_ARG;
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      fd::train::qkv_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kQkvBwdSmem);
+  if (attr != cudaSuccess) return FD_ERR_CUDA;
   fd_trainer tr = new (std::nothrow) fd_trainer_s;
   if (tr == nullptr) return FD_ERR_OOM;
   tr->cfg = *cfg;
@@ -1151,36 +851,36 @@ fd_status fd_train_create(const fd_config* cfg, fd_weights w, int chunks, fd_tra
     tr->xT = dalloc<bf16>(tr, static_cast<size_t>(MB) * tr->cin, ok);
   }
   tr->dqkv16 = dalloc<bf16>(tr, wide, ok);
-  tr->e = dalloc<float>(tr, static_cast<size_t>(MB) * tr->rt * D, ok);
   tr->z1 = dalloc<float>(tr, static_cast<size_t>(MR) * D, ok);
   tr->F = dalloc<float>(tr, static_cast<size_t>(MR) * tr->Cr, ok);
-  tr->dF = dalloc<float>(tr, static_cast<size_t>(MR) * tr->Cr, ok);
-  tr->loss_blocks = static_cast<int>((static_cast<long long>(MR) * tr->Cr + 255) / 256);
-  tr->loss_part = dalloc<float>(tr, tr->loss_blocks, ok);
+  tr->loss_part = dalloc<float>(
+      tr,
+      static_cast<size_t>((MR + fd::train::kRowBlock - 1) / fd::train::kRowBlock) *
+          ((tr->Cr + 1023) / 1024),
+      ok);
   if (materialised) tr->S = dalloc<float>(tr, RK, ok);
   tr->delta = dalloc<float>(tr, static_cast<size_t>(Mmax) * tr->N, ok);
-  {
-    const size_t R = fd::train::kColsumRows;
-    const size_t widest = std::max({D, tr->Dz, QO, NQ, tr->rt * D, tr->Cr});
-    tr->colsum_elems = std::max((static_cast<size_t>(Mmax) * tr->N + R - 1) / R * 64,
-                                (static_cast<size_t>(Mmax) + R - 1) / R * widest);
-    tr->colsum_part = dalloc<float>(tr, tr->colsum_elems, ok);
+  {  // partial rows of the column sums: per kRowBlock rows, per kNormRows rows and group, per
+     // kQkvRows rows (and kQkvSlots slots, 128 columns)
+    using namespace fd::train;
+    const size_t m = Mmax, slots = tr->N + 2 * G;
+    tr->part_elems = std::max({(m + kRowBlock - 1) / kRowBlock *
+                                   std::max({tr->Dz, tr->rt * D, tr->Cr, D}),
+                               (m + kNormRows - 1) / kNormRows * norm_groups(D) * D,
+                               m / kQkvRows * QO,
+                               m / kQkvRows * ((slots + kQkvSlots - 1) / kQkvSlots) * 128});
+    tr->part_a = dalloc<float>(tr, tr->part_elems, ok);
+    tr->part_b = dalloc<float>(tr, tr->part_elems, ok);
   }
   tr->dq2 = dalloc<float>(tr, static_cast<size_t>(Mmax) * NQ, ok);
   tr->dk2 = dalloc<float>(tr, static_cast<size_t>(G) * Mmax * 64, ok);
   tr->dv1 = dalloc<float>(tr, static_cast<size_t>(G) * Mmax * 64, ok);
-  tr->dqkv = dalloc<float>(tr, static_cast<size_t>(Mmax) * QO, ok);
-  tr->tq = dalloc<float>(tr, static_cast<size_t>(Mmax) * tr->N * 64, ok);
-  tr->tk = dalloc<float>(tr, static_cast<size_t>(Mmax) * G * 64, ok);
-  tr->tv = dalloc<float>(tr, static_cast<size_t>(Mmax) * G * 64, ok);
   tr->gA = dalloc<float>(tr, wide, ok);
   tr->gB = dalloc<float>(tr, wide, ok);
   tr->gC = dalloc<float>(tr, wide, ok);
-  tr->tbuf = dalloc<float>(tr, static_cast<size_t>(Mmax) * D, ok);
   if (tr->cin % 64) tr->gtmp = dalloc<float>(tr, static_cast<size_t>(D) * tr->cin, ok);
   if (tr->gated) {
-    tr->dz32 = dalloc<float>(tr, static_cast<size_t>(Mmax) * tr->Dz, ok);
-    tr->dwz = dalloc<float>(tr, static_cast<size_t>(tr->Dz) * (D + 1), ok);
+    tr->dwz = dalloc<float>(tr, static_cast<size_t>(tr->Dz) * D, ok);
   }
   // transposed weights [in][out] for the input gradients dX = dY W
   auto wT = [&](size_t entry, int n_out, int n_in) -> bf16* {
@@ -1248,12 +948,9 @@ fd_status fd_train_step(fd_trainer tr, const float* latents, const float* target
   // final norm and temporal upsampling (Eq. temporal_upsample): channel block tau -> frame tau
   const float* hBo = tr->sB.h[tr->nb];
   r.rmsnorm(hBo, r.wf(eF), MB, tr->y16);
-  r.gemm(FD_TK_LINEAR, fd::EPI_F32, MB, rt * D, D, tr->y16, D, r.wb(eF + 1), D, r.wf(eF + 2), tr->e, rt * D);
-  if (r.begin(FD_TK_POINTWISE)) {
-    const long long n = static_cast<long long>(MB) * rt * D;
-    fd::train::tup_permute_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(
-        tr->e, tr->T, rt, tr->Lp, D, 0, tr->sR.h[0], nullptr);
-    r.check(cudaGetLastError());
+  if (r.begin(FD_TK_LINEAR)) {
+    r.check(fd::gemm_tup(MB, rt, tr->Lp, D, tr->y16, r.wb(eF + 1), r.wf(eF + 2), tr->sR.h[0],
+                         tr->err, r.s));
     r.end();
   }
   for (int b = 0; b < tr->nr; ++b)
@@ -1263,8 +960,9 @@ fd_status fd_train_step(fd_trainer tr, const float* latents, const float* target
   r.rmsnorm(hRo, r.wf(eH), MR, tr->yh16);
   r.gemm(FD_TK_LINEAR, fd::EPI_F32, MR, D, D, tr->yh16, D, r.wb(eH + 1), D, r.wf(eH + 2), tr->z1, D);
   if (r.begin(FD_TK_POINTWISE)) {
-    const long long n = static_cast<long long>(MR) * D;
-    fd::train::gelu_fwd_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(tr->z1, n, tr->a1);
+    const long long n4 = static_cast<long long>(MR) * D / 4;
+    fd::train::gelu_fwd_kernel<<<blocks_for(n4, 256), 256, 0, r.s>>>(
+        reinterpret_cast<const float4*>(tr->z1), n4, reinterpret_cast<uint2*>(tr->a1));
     r.check(cudaGetLastError());
     r.end();
   }
@@ -1274,60 +972,62 @@ fd_status fd_train_step(fd_trainer tr, const float* latents, const float* target
   const double total = (static_cast<double>(tr->T - 1) * rt + first) * tr->Cout * tr->gh *
                        tr->rs * tr->gw * tr->rs;
   const float inv_total = static_cast<float>(1.0 / total);
-  if (r.begin(FD_TK_POINTWISE)) {
-    fd::train::l1_head_kernel<<<tr->loss_blocks, 256, 0, r.s>>>(
-        tr->F, targets, tr->T, rt, first, tr->Lp, tr->L, tr->gh, tr->gw, tr->Cout, tr->rs,
-        inv_total, tr->dF, tr->loss_part);
-    r.check(cudaGetLastError());
-    r.end();
-  }
-  if (r.begin(FD_TK_POINTWISE)) {
-    fd::train::finish_loss_kernel<<<1, fd::train::kLossThreads, 0, r.s>>>(tr->loss_part,
-                                                                         tr->loss_blocks, inv_total,
-                                                     loss);
-    r.check(cudaGetLastError());
-    r.end();
+  float* g = grads;
+  using fd::train::kRowBlock;
+  {
+    const int parts = (MR + kRowBlock - 1) / kRowBlock, strips = (tr->Cr + 1023) / 1024;
+    if (r.room(parts, tr->Cr) && r.begin(FD_TK_POINTWISE)) {
+      const fd::train::PixelGrid pg{tr->T, rt, first, tr->Lp, tr->L, tr->gh, tr->gw, tr->Cout,
+                                    tr->rs, inv_total};
+      fd::train::l1_head4_kernel<<<dim3(strips, parts), 256, 0, r.s>>>(
+          tr->F, targets, pg, nullptr, tr->dy16, tr->part_a, tr->loss_part);
+      r.check(cudaGetLastError());
+      fd::train::finish_loss_kernel<<<1, fd::train::kLossThreads, 0, r.s>>>(
+          tr->loss_part, parts * strips, inv_total, loss);
+      r.check(cudaGetLastError());
+      r.sum_parts({{tr->part_a, parts, tr->Cr, tr->Cr, 0, r.grad(g, eH + 4)}});
+      r.end();
+    }
   }
   // ---- backward
-  float* g = grads;
   // head layer 2
-  r.bf(tr->dF, static_cast<long long>(MR) * tr->Cr, tr->dy16);
   r.gemm(FD_TK_DGRAD, fd::EPI_F32, MR, D, tr->Cr, tr->dy16, tr->Cr, tr->t_head2, tr->Cr, nullptr, tr->gC, D);
   r.wgrad(tr->dy16, tr->Cr, tr->a1, D, MR, r.grad(g, eH + 3));
-  r.colsum(tr->dF, MR, tr->Cr, tr->Cr, r.grad(g, eH + 4));
   // head layer 1 (GELU')
-  if (r.begin(FD_TK_POINTWISE)) {
-    const long long n = static_cast<long long>(MR) * D;
-    fd::train::gelu_bwd_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(tr->z1, tr->gC, n, tr->gC,
-                                                                      tr->dqkv16);
-    r.check(cudaGetLastError());
-    r.end();
-  }
+  r.gelu_bwd(tr->z1, tr->gC, MR, D, tr->dqkv16, r.grad(g, eH + 2));
   r.gemm(FD_TK_DGRAD, fd::EPI_F32, MR, D, D, tr->dqkv16, D, tr->t_head1, D, nullptr, tr->gA, D);
   r.wgrad(tr->dqkv16, D, tr->yh16, D, MR, r.grad(g, eH + 1));
-  r.colsum(tr->gC, MR, D, D, r.grad(g, eH + 2));
+  // the gradient of a block's second MLP bias: the column sums of the block's output gradient
+  auto mlp_bias = [&](size_t e0, int b) {
+    return r.grad(g, e0 + static_cast<size_t>(b) * kBlockEntries + kM2B);
+  };
   // the head's RMSNorm
-  r.rmsnorm_bwd(hRo, r.wf(eH), tr->gA, nullptr, MR, tr->gB, r.grad(g, eH));
+  r.rmsnorm_bwd(hRo, r.wf(eH), tr->gA, nullptr, MR, tr->gB, tr->dy16, r.grad(g, eH),
+                tr->nr > 0 ? mlp_bias(eR, tr->nr - 1) : nullptr);
   for (int b = tr->nr - 1; b >= 0; --b)
-    block_bwd(r, tr->sR, b, eR + static_cast<size_t>(b) * kBlockEntries, tr->tR[b], g);
+    block_bwd(r, tr->sR, b, eR + static_cast<size_t>(b) * kBlockEntries, tr->tR[b], g,
+              b > 0 ? mlp_bias(eR, b - 1) : nullptr);
   // temporal upsampling: refined frame tau back to channel block tau
-  if (r.begin(FD_TK_POINTWISE)) {
-    const long long n = static_cast<long long>(MB) * rt * D;
-    fd::train::tup_permute_kernel<<<blocks_for(n, 256), 256, 0, r.s>>>(
-        tr->gB, tr->T, rt, tr->Lp, D, 1, tr->gC, tr->dqkv16);
-    r.check(cudaGetLastError());
-    r.end();
+  {
+    const int parts = (MB + kRowBlock - 1) / kRowBlock, cols = rt * D;
+    if (r.room(parts, cols) && r.begin(FD_TK_POINTWISE)) {
+      fd::train::tup_bwd_kernel<<<dim3((cols + 1023) / 1024, parts), 256, 0, r.s>>>(
+          tr->gB, MB, rt, tr->Lp, D, tr->dqkv16, tr->part_a);
+      r.check(cudaGetLastError());
+      r.sum_parts({{tr->part_a, parts, cols, cols, 0, r.grad(g, eF + 2)}});
+      r.end();
+    }
   }
   r.gemm(FD_TK_DGRAD, fd::EPI_F32, MB, D, rt * D, tr->dqkv16, rt * D, tr->t_tup, rt * D, nullptr, tr->gA, D);
   r.wgrad(tr->dqkv16, rt * D, tr->y16, D, MB, r.grad(g, eF + 1));
-  r.colsum(tr->gC, MB, rt * D, rt * D, r.grad(g, eF + 2));
-  r.rmsnorm_bwd(hBo, r.wf(eF), tr->gA, nullptr, MB, tr->gB, r.grad(g, eF));
+  r.rmsnorm_bwd(hBo, r.wf(eF), tr->gA, nullptr, MB, tr->gB, tr->dy16, r.grad(g, eF),
+                mlp_bias(eB, tr->nb - 1));
+  // the first block's input gradient sums to the patch-embedding's bias gradient
   for (int b = tr->nb - 1; b >= 0; --b)
-    block_bwd(r, tr->sB, b, eB + static_cast<size_t>(b) * kBlockEntries, tr->tB[b], g);
-  // patch-embedding: weight and bias gradients only
-  r.bf(tr->gB, static_cast<long long>(MB) * D, tr->dy16);
+    block_bwd(r, tr->sB, b, eB + static_cast<size_t>(b) * kBlockEntries, tr->tB[b], g,
+              b > 0 ? mlp_bias(eB, b - 1) : r.grad(g, 1));
+  // patch-embedding: the weight gradient
   r.wgrad(tr->dy16, D, tr->x0, tr->cin, MB, r.grad(g, 0));
-  r.colsum(tr->gB, MB, D, D, r.grad(g, 1));
   return r.ok ? FD_OK : FD_ERR_CUDA;
 }
 
@@ -1354,19 +1054,40 @@ fd_status fd_op_rmsnorm_bwd(const float* x, const float* g, const float* dy, int
                             float eps, float* dx, float* dg, float* work, void* stream) {
   if (!x || !g || !dy || !dx || !dg || !work || M < 1 || D < 1 || D > 65536)
     return FD_ERR_INVALID_ARG;
+  using namespace fd::train;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  fd::train::rmsnorm_bwd_kernel<<<(M + 7) / 8, 256, 0, s>>>(x, g, dy, nullptr, M, D, eps, dx,
-                                                            work);
+  // partial rows of dg in the caller's scratch (at most M of them)
+  const int blocks = (M + kNormRows - 1) / kNormRows;
+  int groups = norm_groups(D);
+  if (blocks * groups > M) groups = 1;
+  const bool vec = D % 4 == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy) |
+                                   reinterpret_cast<uintptr_t>(dx)) & 15u) == 0;
+  if (vec)
+    rmsnorm_bwd_kernel<4><<<blocks, 256, 0, s>>>(x, g, dy, nullptr, M, D, eps, groups, dx, nullptr,
+                                                work, nullptr);
+  else
+    rmsnorm_bwd_kernel<1><<<blocks, 256, 0, s>>>(x, g, dy, nullptr, M, D, eps, groups, dx, nullptr,
+                                                work, nullptr);
   if (cudaGetLastError() != cudaSuccess) return FD_ERR_CUDA;
-  fd::train::colsum_kernel<<<(D + 127) / 128, 128, 0, s>>>(work, M, D, D, dg);
+  SumJobs js{};
+  js.job[0] = {work, blocks * groups, D, D, 0, dg};
+  sum_parts_kernel<<<dim3((D + 31) / 32, 1), dim3(32, kSumRows), 0, s>>>(js);
   return cudaGetLastError() == cudaSuccess ? FD_OK : FD_ERR_CUDA;
 }
 
 fd_status fd_op_gelu_bwd(const float* z, const float* da, int64_t n, float* dz, void* dz_bf16,
                          void* stream) {
   if (!z || !da || !dz || !dz_bf16 || n < 1) return FD_ERR_INVALID_ARG;
-  fd::train::gelu_bwd_kernel<<<blocks_for(n, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      z, da, n, dz, static_cast<bf16*>(dz_bf16));
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  bf16* const dz16 = static_cast<bf16*>(dz_bf16);
+  const bool vec =
+      n % 4 == 0 && ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(da) |
+                      reinterpret_cast<uintptr_t>(dz)) & 15u) == 0 &&
+      (reinterpret_cast<uintptr_t>(dz16) & 7u) == 0;
+  if (vec)
+    fd::train::gelu_bwd_kernel<4><<<blocks_for(n / 4, 256), 256, 0, s>>>(z, da, n, dz, dz16);
+  else
+    fd::train::gelu_bwd_kernel<1><<<blocks_for(n, 256), 256, 0, s>>>(z, da, n, dz, dz16);
   return cudaGetLastError() == cudaSuccess ? FD_OK : FD_ERR_CUDA;
 }
 
@@ -1382,11 +1103,23 @@ fd_status fd_op_l1_pixel_bwd(const float* F, const float* target, int frames, in
   const int blocks = static_cast<int>((n + 255) / 256);
   const float inv_total = static_cast<float>(1.0 / static_cast<double>(n));
   // one chunk of `frames` refined frames, rows unpadded (Lp = L)
-  fd::train::l1_head_kernel<<<blocks, 256, 0, s>>>(F, target, 1, frames, frames, L, L, grid_h,
-                                                   grid_w, channels, rs, inv_total, dF, work);
+  const fd::train::PixelGrid pg{1, frames, frames, L, L, grid_h, grid_w, channels, rs, inv_total};
+  const int cols = channels * rs * rs;
+  const bool vec = rs % 4 == 0 && ((reinterpret_cast<uintptr_t>(F) |
+                                    reinterpret_cast<uintptr_t>(target) |
+                                    reinterpret_cast<uintptr_t>(dF)) & 15u) == 0;
+  int parts = blocks;
+  if (vec) {  // no more partial sums than the caller's scratch holds: a row has cols >= 16 elements
+    const int strips = (cols + 1023) / 1024;
+    const int rows = (frames * L + fd::train::kRowBlock - 1) / fd::train::kRowBlock;
+    parts = strips * rows;
+    fd::train::l1_head4_kernel<<<dim3(strips, rows), 256, 0, s>>>(F, target, pg, dF, nullptr,
+                                                                 nullptr, work);
+  } else {
+    fd::train::l1_head_kernel<<<blocks, 256, 0, s>>>(F, target, pg, dF, work);
+  }
   if (cudaGetLastError() != cudaSuccess) return FD_ERR_CUDA;
-  fd::train::finish_loss_kernel<<<1, fd::train::kLossThreads, 0, s>>>(work, blocks, inv_total,
-                                                                       loss);
+  fd::train::finish_loss_kernel<<<1, fd::train::kLossThreads, 0, s>>>(work, parts, inv_total, loss);
   return cudaGetLastError() == cudaSuccess ? FD_OK : FD_ERR_CUDA;
 }
 

@@ -1362,6 +1362,32 @@ cudaError_t gemm_view(int epi, int M, int N, int K, const __nv_bfloat16* A, int 
   return launch_gemm(ta, tb, to, to, to, p, t.bn, t.pair, num_sms(), s);
 }
 
+cudaError_t gemm_tup(int M, int rt, int Lp, int D, const __nv_bfloat16* y, const __nv_bfloat16* W,
+                     const float* bias, float* out, int* err, cudaStream_t s) {
+  if (M < 1 || rt < 1 || Lp < 1 || M % Lp || D % 32 || !aligned16(y) || !aligned16(W) ||
+      !aligned16(bias) || !aligned16(out))
+    return cudaErrorInvalidValue;
+  const int N = rt * D;
+  const TileChoice t = pick_tile(M, N, D, 32, false);
+  CUtensorMap ta, tb, to;
+  if (!tmap_bf16(&ta, y, D, M, static_cast<uint64_t>(D) * 2, 64, 128) ||
+      !tmap_bf16(&tb, W, D, N, static_cast<uint64_t>(D) * 2, 64, t.pair ? t.bn / 2 : t.bn) ||
+      !tmap_out_tup(&to, out, D, Lp, rt, M / Lp))
+    return cudaErrorInvalidValue;
+  GemmParams p{};
+  p.M = M;
+  p.N = N;
+  p.K = D;
+  p.epi = EPI_TUP;
+  p.bias = bias;
+  p.out_f32 = out;
+  p.ld_out = D;
+  p.tup_tokens = Lp;
+  p.tup_hidden = D;
+  p.err = err;
+  return launch_gemm(ta, tb, to, to, to, p, t.bn, t.pair, num_sms(), s);
+}
+
 cudaError_t gemm_wgrad(int n_out, int n_in, int rows, const __nv_bfloat16* dY,
                        const __nv_bfloat16* X, const float* zero_bias, float* dW, int* err,
                        cudaStream_t s) {
