@@ -63,77 +63,6 @@ __global__ void transpose_kernel(const T* __restrict__ x, int rows, int cols, in
   }
 }
 
-// RMS over the 64 values of one head with gain g
-__device__ __forceinline__ void head_rms(float (&v)[kDh], const float* g, float eps) {
-  float ss = 0.f;
-#pragma unroll
-  for (int j = 0; j < kDh; ++j) ss = fmaf(v[j], v[j], ss);
-  const float r = rsqrtf(ss / kDh + eps);
-#pragma unroll
-  for (int j = 0; j < kDh; ++j) v[j] = v[j] * r * g[j];
-}
-
-// QKV forward of every row: slot < N query heads, then G key groups, then G value groups.
-// q2 = RoPE(q0) (RMS with g2 first when qk_norm), k2 = RoPE(RMS(k0; gk)), v1 = RMS(v0; g2)
-// (v0 when qk_norm). Outputs: q2 bf16 head-major per chunk of Pc rows, [M / Pc][N][Pc][64]
-// (the rows of one chunk's heads of a KV group are then contiguous), k2 / v1 bf16 [G][M][64].
-// With qr non-null, also: q rows bf16 [M][N 64] (the attention kernel's layout), and the
-// real tokens' K bf16 [G][pitch][64] and V^T fp16 [G][64][pitch] without the padding rows
-// (chunk c's Lu = Pc / Lp * L keys at c Lu ...), the keys of the fused band attention.
-__global__ void qkv_fwd_kernel(const float* __restrict__ qkv, int M, int Pc, int Lp, int L,
-                               int gw, int N, int G, int qk_norm, const float* __restrict__ gk,
-                               const float* __restrict__ g2, float eps, Rope rp,
-                               bf16* __restrict__ q2, bf16* __restrict__ k2,
-                               bf16* __restrict__ v1, bf16* __restrict__ qr,
-                               bf16* __restrict__ ku, __half* __restrict__ vtu, int pitch) {
-  const int slots = N + 2 * G;
-  const long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-  if (idx >= static_cast<long long>(M) * slots) return;
-  const int row = static_cast<int>(idx / slots), slot = static_cast<int>(idx % slots);
-  const int f = row / Lp, l = min(row % Lp, L - 1);  // padding rows take a real token's angles
-  const int gy = l / gw, gx = l % gw;
-  float v[kDh];
-  const float* src = qkv + static_cast<size_t>(row) * slots * kDh + slot * kDh;
-#pragma unroll
-  for (int j = 0; j < kDh; ++j) v[j] = src[j];
-  const bool is_q = slot < N, is_k = !is_q && slot < N + G;
-  if (is_k) head_rms(v, gk, eps);
-  else if (is_q ? qk_norm != 0 : qk_norm == 0) head_rms(v, g2, eps);
-  bf16* dst;
-  if (is_q) dst = q2 + (static_cast<size_t>(row / Pc * N + slot) * Pc + row % Pc) * kDh;
-  else if (is_k) dst = k2 + (static_cast<size_t>(slot - N) * M + row) * kDh;
-  else dst = v1 + (static_cast<size_t>(slot - N - G) * M + row) * kDh;
-  if (is_q || is_k) {
-#pragma unroll
-    for (int i = 0; i < kDh / 2; ++i) {
-      const float2 cs = rope_cs(rp, i, f, gy, gx);
-      const float a = v[2 * i], b = v[2 * i + 1];
-      v[2 * i] = a * cs.x - b * cs.y;
-      v[2 * i + 1] = a * cs.y + b * cs.x;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < kDh; ++j) dst[j] = __float2bfloat16_rn(v[j]);
-  if (qr == nullptr) return;
-  if (is_q) {
-    bf16* d = qr + static_cast<size_t>(row) * N * kDh + slot * kDh;
-#pragma unroll
-    for (int j = 0; j < kDh; ++j) d[j] = __float2bfloat16_rn(v[j]);
-    return;
-  }
-  if (row % Lp >= L) return;  // padding rows are no keys
-  const int key = row / Pc * (Pc / Lp * L) + row % Pc / Lp * L + row % Lp;
-  if (is_k) {
-    bf16* d = ku + (static_cast<size_t>(slot - N) * pitch + key) * kDh;
-#pragma unroll
-    for (int j = 0; j < kDh; ++j) d[j] = __float2bfloat16_rn(v[j]);
-  } else {
-    __half* d = vtu + static_cast<size_t>(slot - N - G) * kDh * pitch + key;
-#pragma unroll
-    for (int j = 0; j < kDh; ++j) d[static_cast<size_t>(j) * pitch] = __float2half_rn(v[j]);
-  }
-}
-
 // Band softmax of one (query chunk, KV group): S fp32 [rows][n] (row pitch n), rows = the
 // group's heads x the chunk's rows; column c is a key of a token (c mod Lp < L). P = softmax(S
 // scale) over the valid columns (0 elsewhere) as bf16, and lse = log sum exp(S scale) of each
@@ -315,6 +244,11 @@ double rope_inv_freq(int i, double base) {
 }
 
 constexpr int kQkvBwdSmem = 2 * fd::train::kQkvUnits * fd::train::kQkvPad * 4;
+// + the block's V^T: at most kQkvSlots groups
+int qkv_fwd_smem(int G) {
+  using namespace fd::train;
+  return kQkvUnits * kQkvPad * 4 + std::min(G, kQkvSlots) * kDh * kQkvRows * 2;
+}
 
 // thread groups that share a block's rows in the RMSNorm backward (one for D >= 1024)
 int norm_groups(int D) {
@@ -548,12 +482,14 @@ void block_fwd(Run& r, fd_trainer_s::Stack& st, int b, size_t e0) {
   r.gemm(FD_TK_LINEAR, fd::EPI_F32, M, tr->QO, tr->D, st.u[b], tr->D, r.wb(e0 + kQW), tr->D, r.wf(e0 + kQB),
          st.qkv[b], tr->QO);
   if (r.begin(FD_TK_NORM)) {
-    const fd::train::Rope rp{tr->rope_t, tr->rope_y, tr->rope_x};
-    const long long n = static_cast<long long>(M) * (tr->N + 2 * tr->G);
-    fd::train::qkv_fwd_kernel<<<blocks_for(n, 128), 128, 0, r.s>>>(
-        st.qkv[b], M, st.Pc, tr->Lp, tr->L, tr->gw, tr->N, tr->G, tr->cfg.qk_norm, r.wf(e0 + kKG),
-        r.wf(e0 + kG2), tr->eps, rp, st.q2[b], st.k2[b], st.v1[b], st.band.on ? st.band.qr : nullptr,
-        st.band.k, st.band.vt, st.band.pitch);
+    using namespace fd::train;
+    const Rope rp{tr->rope_t, tr->rope_y, tr->rope_x};
+    const QkvShape sh{M, st.Pc, tr->Lp, tr->L, tr->gw, tr->N, tr->G, tr->cfg.qk_norm};
+    const int slots = tr->N + 2 * tr->G;
+    qkv_fwd_kernel<<<dim3(M / kQkvRows, (slots + kQkvSlots - 1) / kQkvSlots), kQkvUnits,
+                     qkv_fwd_smem(tr->G), r.s>>>(
+        st.qkv[b], sh, r.wf(e0 + kKG), r.wf(e0 + kG2), tr->eps, rp, st.q2[b], st.k2[b], st.v1[b],
+        st.band.on ? st.band.qr : nullptr, st.band.k, st.band.vt, st.band.pitch);
     r.check(cudaGetLastError());
     r.end();
   }
@@ -667,9 +603,12 @@ fd_status fd_train_create(const fd_config* cfg, fd_weights w, int chunks, fd_tra
   // the bf16-valued decoder: GELU or gated-SiLU MLPs, r_t frames per chunk or one from chunk 0
   if (cfg->mlp_fp8) return FD_ERR_CONFIG;
   if (chunks < 1 || chunks > 256) return FD_ERR_INVALID_ARG;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      fd::train::qkv_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kQkvBwdSmem);
-  if (attr != cudaSuccess) return FD_ERR_CUDA;
+  static const cudaError_t attr[2] = {
+      cudaFuncSetAttribute(fd::train::qkv_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           kQkvBwdSmem),
+      cudaFuncSetAttribute(fd::train::qkv_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           qkv_fwd_smem(fd::train::kQkvSlots))};
+  if (attr[0] != cudaSuccess || attr[1] != cudaSuccess) return FD_ERR_CUDA;
   fd_trainer tr = new (std::nothrow) fd_trainer_s;
   if (tr == nullptr) return FD_ERR_OOM;
   tr->cfg = *cfg;

@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// ---------------------------------------------------------------- QKV, backward
+// ---------------------------------------------------------------- QKV
 // RoPE tables (host-computed in double): temporal (cos, sin) [frames][kBandT], row and column
 // [grid][kBandS]
 constexpr int kBandS = kHeadDim / 6;               // pairs per spatial band (10)
@@ -310,13 +310,109 @@ struct QkvShape {
     return slot < N ? static_cast<size_t>(row / Pc * N + slot) * Pc + row % Pc
                     : static_cast<size_t>((slot - N) % G) * M + row;
   }
+  __device__ int key(int row) const {  // position of a token's row among the unpadded keys
+    return (row / Pc * (Pc / Lp) + row % Pc / Lp) * L + row % Lp;
+  }
 };
+
+// RMS over the 64 values of one head with gain g
+__device__ __forceinline__ void head_rms(float (&v)[kDh], const float* g, float eps) {
+  float ss = 0.f;
+#pragma unroll
+  for (int j = 0; j < kDh; ++j) ss = fmaf(v[j], v[j], ss);
+  const float r = rsqrtf(ss / kDh + eps);
+#pragma unroll
+  for (int j = 0; j < kDh; ++j) v[j] = v[j] * r * g[j];
+}
 // One thread does one (row, slot): its 64 values in order, as the sums over a head are. A block
 // stages kQkvBatch rows x up to kQkvSlots slots through shared memory (65 floats per unit: no bank
 // conflicts), so that global memory is read and written in whole lines: a thread reading its own
-// 256 bytes took 136 us forward and 89 us backward on average at 480p. kQkvRows rows per block.
+// 256 bytes took 136 us forward and 89 us backward on average at 480p (36 and 52 staged). kQkvRows rows
+// per block.
 constexpr int kQkvBatch = 4, kQkvSlots = 32, kQkvRows = 16, kQkvPad = 65;
 constexpr int kQkvUnits = kQkvBatch * kQkvSlots;  // threads
+
+// QKV forward: q2 = RoPE(q0) (RMS with g2 first when qk_norm), k2 = RoPE(RMS(k0; gk)),
+// v1 = RMS(v0; g2) (v0 when qk_norm), in bf16. With qr non-null, also: q rows bf16 [M][N 64] (the
+// attention kernel's layout), and the real tokens' K bf16 [G][pitch][64] and V^T fp16
+// [G][64][pitch] without the padding rows (chunk c's Lu = Pc / Lp * L keys at c Lu ...), the keys
+// of the fused band attention. V^T leaves as the block's kQkvRows keys of each dimension.
+__global__ void __launch_bounds__(kQkvUnits)
+    qkv_fwd_kernel(const float* __restrict__ qkv, QkvShape p, const float* __restrict__ gk,
+                   const float* __restrict__ g2, float eps, Rope rp, bf16* __restrict__ q2,
+                   bf16* __restrict__ k2, bf16* __restrict__ v1, bf16* __restrict__ qr,
+                   bf16* __restrict__ ku, __half* __restrict__ vtu, int pitch) {
+  extern __shared__ float sm[];
+  float* const xs = sm;
+  __half* const vts = reinterpret_cast<__half*>(sm + kQkvUnits * kQkvPad);
+  const int slots = p.N + 2 * p.G, s0 = blockIdx.y * kQkvSlots;
+  const int sc = min(kQkvSlots, slots - s0), units = kQkvBatch * sc;
+  const int v0 = max(p.N + p.G, s0);  // first V slot of the block
+  const int tid = threadIdx.x;
+  for (int b = 0; b < kQkvRows / kQkvBatch; ++b) {
+    const int row0 = blockIdx.x * kQkvRows + b * kQkvBatch;
+    for (int i = tid; i < units * 16; i += kQkvUnits) {
+      const int u = i / 16, j = i % 16 * 4;
+      const float4 x = *reinterpret_cast<const float4*>(
+          qkv + (static_cast<size_t>(row0 + u / sc) * slots + s0 + u % sc) * kDh + j);
+      float* px = xs + u * kQkvPad + j;
+      px[0] = x.x; px[1] = x.y; px[2] = x.z; px[3] = x.w;
+    }
+    __syncthreads();
+    if (tid < units) {
+      const int row = row0 + tid / sc, slot = s0 + tid % sc;
+      const int f = row / p.Lp, l = min(row % p.Lp, p.L - 1);  // padding rows: a real token's angles
+      const int gy = l / p.gw, gx = l % p.gw;
+      const bool is_q = slot < p.N, is_k = !is_q && slot < p.N + p.G;
+      float v[kDh];
+      float* px = xs + tid * kQkvPad;
+#pragma unroll
+      for (int j = 0; j < kDh; ++j) v[j] = px[j];
+      if (is_k) head_rms(v, gk, eps);
+      else if (is_q ? p.qk_norm != 0 : p.qk_norm == 0) head_rms(v, g2, eps);
+      if (is_q || is_k) {
+#pragma unroll
+        for (int i = 0; i < kDh / 2; ++i) {
+          const float2 cs = rope_cs(rp, i, f, gy, gx);
+          const float a = v[2 * i], c = v[2 * i + 1];
+          v[2 * i] = a * cs.x - c * cs.y;
+          v[2 * i + 1] = a * cs.y + c * cs.x;
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kDh; ++j) px[j] = v[j];
+    }
+    __syncthreads();
+    for (int i = tid; i < units * 8; i += kQkvUnits) {  // eight values (16 bytes) each
+      const int u = i / 8, j = i % 8 * 8, row = row0 + u / sc, slot = s0 + u % sc;
+      const float* px = xs + u * kQkvPad + j;
+      const uint2 lo = pack4(px[0], px[1], px[2], px[3]), hi = pack4(px[4], px[5], px[6], px[7]);
+      const uint4 w = make_uint4(lo.x, lo.y, hi.x, hi.y);
+      const bool is_q = slot < p.N, is_k = !is_q && slot < p.N + p.G;
+      bf16* dst = is_q ? q2 : (is_k ? k2 : v1);
+      *reinterpret_cast<uint4*>(dst + p.head_row(row, slot) * kDh + j) = w;
+      if (qr == nullptr) continue;
+      if (is_q) {
+        *reinterpret_cast<uint4*>(qr + (static_cast<size_t>(row) * p.N + slot) * kDh + j) = w;
+      } else if (!is_k) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          vts[((slot - v0) * kDh + j + k) * kQkvRows + row % kQkvRows] = __float2half_rn(px[k]);
+      } else if (row % p.Lp < p.L) {  // padding rows are no keys
+        *reinterpret_cast<uint4*>(
+            ku + (static_cast<size_t>(slot - p.N) * pitch + p.key(row)) * kDh + j) = w;
+      }
+    }
+    __syncthreads();
+  }
+  if (qr == nullptr) return;
+  const int r0 = blockIdx.x * kQkvRows, nv = s0 + sc - v0;  // V slots of the block
+  for (int i = tid; i < nv * kDh * kQkvRows; i += kQkvUnits) {
+    const int r = r0 + i % kQkvRows, d = i / kQkvRows;  // d: dimension of group v0 - N - G + d / 64
+    if (r % p.Lp < p.L)
+      vtu[(static_cast<size_t>(v0 - p.N - p.G) * kDh + d) * pitch + p.key(r)] = vts[i];
+  }
+}
 
 // RMS over one head, backward: x the pre-norm values in shared memory, overwritten by the gain's
 // gradient terms dy x r; dy the gradient of the normed output, overwritten by dx
