@@ -22,7 +22,7 @@
 // dV one chain per (query chunk, hs heads), the chains added in fp32 in that order. No atomics.
 //
 // Warps: 0 TMA (the CTA's own two tiles once, then the streamed pairs into a ring), 1 MMA issue,
-// 2-9 element-wise: two warps per 32 TMEM lanes, 64 columns each; a warp takes S and dP into
+// 2-17 element-wise: four warps per 32 TMEM lanes, 32 columns each; a warp takes S and dP into
 // registers and releases them at once, so that the next block's S and dP run under its arithmetic.
 #include "fd_internal.h"
 #include "fd_ptx.cuh"
@@ -37,20 +37,32 @@ constexpr int kOffY = 2 * kTile;  // ring of streamed pairs: K, V or Q, dO
 constexpr int kOffL = kOffY + kStages * 2 * kTile;  // ring of lse[128], delta[128] (dK / dV)
 constexpr int kOffBar = kOffL + kStages * 1024;
 constexpr int kSmem = kOffBar + 256;
-constexpr int kThreads = 320;
-constexpr int kElemWarps = 8;
+constexpr int kElemWarps = 16;
+constexpr int kThreads = 64 + 32 * kElemWarps;
 constexpr uint32_t kColS = 0, kColDp = 128, kColDs = 256, kColP = 320, kColAcc = 384;
 enum Bar { kXFull, kFull, kEmpty = kFull + kStages, kSReady = kEmpty + kStages, kSFree, kPFull,
            kPFree, kAccDone, kAccFree, kDone, kNumBars };
 static_assert(kNumBars * 8 + 8 <= 256 && kSmem <= 227 * 1024, "shared memory");
 }  // namespace attn_bwd
 
-// P and dS of one element: the softmax and its derivative, given the row's log-sum-exp (+inf: a
-// padding row, P = 0) and delta
-__device__ __forceinline__ void score_grad(float s, float dp, float lse, float delta, float& pr,
-                                           float& ds) {
-  pr = expf(fmaf(s, 0.125f, -lse));
-  ds = pr * (dp - delta) * 0.125f;
+// P and dS of two elements: the softmax and its derivative, given each one's row log-sum-exp
+// (negated; -inf for a padding row: P = 0) and delta (negated). Packed fp32 pairs, each operation
+// rounded as its scalar form.
+__device__ __forceinline__ void score_grad2(uint32_t s0, uint32_t s1, uint32_t d0, uint32_t d1,
+                                            uint64_t nlse, uint64_t ndelta, float (&pr)[2],
+                                            float (&ds)[2]) {
+  const uint64_t scale = pack_f32x2(0.125f, 0.125f);
+  uint64_t x = pack_f32x2(__uint_as_float(s0), __uint_as_float(s1));
+  uint64_t y = pack_f32x2(__uint_as_float(d0), __uint_as_float(d1));
+  asm("fma.rn.f32x2 %0, %0, %1, %2;" : "+l"(x) : "l"(scale), "l"(nlse));
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
+  pr[0] = expf(a);
+  pr[1] = expf(b);
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(y) : "l"(ndelta));
+  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(y) : "l"(pack_f32x2(pr[0], pr[1])));
+  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(y) : "l"(scale));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(ds[0]), "=f"(ds[1]) : "l"(y));
 }
 
 // The unit of a CTA. dQ: query rows q0 .. of head h, chunk i; keys k0 .. of the window. dK / dV:
@@ -197,8 +209,12 @@ __global__ void __launch_bounds__(attn_bwd::kThreads, 1)
         tc_fence_after();
         const uint64_t y = dy + static_cast<uint64_t>(gst) * 2 * kT;
         if (elect_one()) {
-          mma8_bf16_ts_mn(tmem + kColAcc, tmem + kColDs, y, id_g, first ? 0u : 1u);
-          if (KV) mma8_bf16_ts_mn(tmem + kColAcc + 64, tmem + kColP, y + kT, id_g, first ? 0u : 1u);
+          mma4_bf16_ts_mn(tmem + kColAcc, tmem + kColDs, y, id_g, first ? 0u : 1u);
+          mma4_bf16_ts_mn(tmem + kColAcc, tmem + kColDs + 32, y + kT / 2, id_g, 1u);
+          if (KV) {
+            mma4_bf16_ts_mn(tmem + kColAcc + 64, tmem + kColP, y + kT, id_g, first ? 0u : 1u);
+            mma4_bf16_ts_mn(tmem + kColAcc + 64, tmem + kColP + 32, y + kT + kT / 2, id_g, 1u);
+          }
           mma_commit(bar(kPFree));
           mma_commit(bar(kEmpty + gst));
           if (last) mma_commit(bar(kAccDone));
@@ -214,13 +230,14 @@ __global__ void __launch_bounds__(attn_bwd::kThreads, 1)
     const int quarter = warp & 3, hc = (warp - 2) >> 2;
     const int row = quarter * 32 + lane;  // TMEM lane: query row (dQ) or key (dK / dV)
     const uint32_t lanes = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
-    float lse = 0.f, delta = 0.f;
+    uint64_t nlse = 0, ndelta = 0;
     bool key_live = true;
     if constexpr (KV) {
       key_live = (key + row) % p.Lp < p.L;
     } else {
-      lse = __ldg(p.lse + xrow + row);
-      delta = __ldg(p.delta + xrow + row);
+      const float a = -__ldg(p.lse + xrow + row), b = -__ldg(p.delta + xrow + row);
+      nlse = pack_f32x2(a, a);
+      ndelta = pack_f32x2(b, b);
     }
     const bool all_live = __all_sync(0xffffffffu, key_live);
     int st = 0, in_group = 0, groups = 0;
@@ -230,69 +247,57 @@ __global__ void __launch_bounds__(attn_bwd::kThreads, 1)
       if (KV && !mbar_wait_warp(bar(kFull + st), ph, p.err, ERR_WAIT_TMA)) break;
       if (!mbar_wait_warp(bar(kSReady), j & 1, p.err, ERR_WAIT_MMA)) break;
       tc_fence_after();
-      uint32_t s[2][32], d[2][32];
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        tmem_ld_32x32b_x32(lanes + kColS + 64u * hc + 32u * c, s[c]);
-        tmem_ld_32x32b_x32(lanes + kColDp + 64u * hc + 32u * c, d[c]);
-      }
+      uint32_t s[32], d[32];
+      tmem_ld_32x32b_x32(lanes + kColS + 32u * hc, s);
+      tmem_ld_32x32b_x32(lanes + kColDp + 32u * hc, d);
       tmem_ld_wait();
       tc_fence_before();
       __syncwarp();
       if (elect_one()) mbar_arrive(bar(kSFree));
-      uint32_t pd[32], pp[KV ? 32 : 1];
+      uint32_t pd[16], pp[KV ? 16 : 1];
 #pragma unroll
-      for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-          float4 l4, d4;
-          if constexpr (KV) {  // the block's lse and delta by column, the same for every lane
-            const float4* q = reinterpret_cast<const float4*>(smem + kOffL + st * 1024) + 16 * hc +
-                              8 * c + e / 4;
-            l4 = q[0];
-            d4 = q[32];
-          } else {
-            l4 = make_float4(lse, lse, lse, lse);
-            d4 = make_float4(delta, delta, delta, delta);
-          }
-          float pr[4], ds[4];
-          score_grad(__uint_as_float(s[c][e]), __uint_as_float(d[c][e]), l4.x, d4.x, pr[0], ds[0]);
-          score_grad(__uint_as_float(s[c][e + 1]), __uint_as_float(d[c][e + 1]), l4.y, d4.y, pr[1],
-                     ds[1]);
-          score_grad(__uint_as_float(s[c][e + 2]), __uint_as_float(d[c][e + 2]), l4.z, d4.z, pr[2],
-                     ds[2]);
-          score_grad(__uint_as_float(s[c][e + 3]), __uint_as_float(d[c][e + 3]), l4.w, d4.w, pr[3],
-                     ds[3]);
-          const int k = 16 * c + e / 2;
-          pd[k] = pack_bf16x2(ds[0], ds[1]);
-          pd[k + 1] = pack_bf16x2(ds[2], ds[3]);
-          if constexpr (KV) {
-            pp[k] = pack_bf16x2(pr[0], pr[1]);
-            pp[k + 1] = pack_bf16x2(pr[2], pr[3]);
-          }
+      for (int e = 0; e < 32; e += 4) {
+        uint64_t nl[2] = {nlse, nlse}, nd[2] = {ndelta, ndelta};
+        if constexpr (KV) {  // the block's lse and delta by column, the same for every lane
+          const float4* q =
+              reinterpret_cast<const float4*>(smem + kOffL + st * 1024) + 8 * hc + e / 4;
+          const float4 l4 = q[0], d4 = q[32];
+          nl[0] = pack_f32x2(-l4.x, -l4.y);
+          nl[1] = pack_f32x2(-l4.z, -l4.w);
+          nd[0] = pack_f32x2(-d4.x, -d4.y);
+          nd[1] = pack_f32x2(-d4.z, -d4.w);
         }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          float pr[2], ds[2];
+          score_grad2(s[e + 2 * k], s[e + 2 * k + 1], d[e + 2 * k], d[e + 2 * k + 1], nl[k], nd[k],
+                      pr, ds);
+          pd[e / 2 + k] = pack_bf16x2(ds[0], ds[1]);
+          if constexpr (KV) pp[e / 2 + k] = pack_bf16x2(pr[0], pr[1]);
+        }
+      }
       // padding keys take no part: their rows (dK / dV) or columns (dQ) are zero
       if constexpr (KV) {
         if (!all_live) {
 #pragma unroll
-          for (int k = 0; k < 32; ++k) {
+          for (int k = 0; k < 16; ++k) {
             pd[k] = key_live ? pd[k] : 0u;
             pp[k] = key_live ? pp[k] : 0u;
           }
         }
       } else {
-        const int live = p.L - kpos - 64 * hc;  // keys among this half's columns
-        if (live < 64) {
+        const int live = p.L - kpos - 32 * hc;  // keys among this warp's columns
+        if (live < 32) {
 #pragma unroll
-          for (int k = 0; k < 32; ++k)
+          for (int k = 0; k < 16; ++k)
             pd[k] = 2 * k + 1 < live ? pd[k] : (2 * k < live ? pd[k] & 0xffffu : 0u);
         }
         kpos = kpos + 128 == p.Lp ? 0 : kpos + 128;
       }
       if (j > 0 && !mbar_wait_warp(bar(kPFree), (j - 1) & 1, p.err, ERR_WAIT_MMA)) break;
       tc_fence_after();
-      tmem_st_32x32b_x32(lanes + kColDs + 32u * hc, pd);
-      if constexpr (KV) tmem_st_32x32b_x32(lanes + kColP + 32u * hc, pp);
+      tmem_st_32x32b_x16(lanes + kColDs + 16u * hc, pd);
+      if constexpr (KV) tmem_st_32x32b_x16(lanes + kColP + 16u * hc, pp);
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
@@ -303,19 +308,19 @@ __global__ void __launch_bounds__(attn_bwd::kThreads, 1)
       }
       if (++in_group < group) continue;
 
-      // the chain's sums: 32 columns per thread, the first chain stored, later ones added
+      // the chain's sums: 16 columns per thread, the first chain stored, later ones added
       in_group = 0;
       if (!mbar_wait_warp(bar(kAccDone), groups & 1, p.err, ERR_WAIT_MMA)) break;
       tc_fence_after();
 #pragma unroll
       for (int a = 0; a < (KV ? 2 : 1); ++a) {
-        uint32_t o[32];
-        tmem_ld_32x32b_x32(lanes + kColAcc + 64u * a + 32u * hc, o);
+        uint32_t o[16];
+        tmem_ld_32x32b_x16(lanes + kColAcc + 64u * a + 16u * hc, o);
         tmem_ld_wait();
         float4* dst = reinterpret_cast<float4*>((a == 0 ? p.out0 : p.out1) +
-                                                static_cast<size_t>(xrow + row) * 64 + 32 * hc);
+                                                static_cast<size_t>(xrow + row) * 64 + 16 * hc);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
+        for (int k = 0; k < 4; ++k) {
           float4 v = make_float4(__uint_as_float(o[4 * k]), __uint_as_float(o[4 * k + 1]),
                                  __uint_as_float(o[4 * k + 2]), __uint_as_float(o[4 * k + 3]));
           if (KV && groups > 0) {
