@@ -23,13 +23,13 @@
 // Warp roles (352 threads):
 //   warp 8        TMA: the two Q tiles of each segment into one of two buffers, K and V^T
 //                 blocks of 128 keys into a 3-stage ring
-//   warps 9 / 10  one thread each issues tile 0's / tile 1's MMAs: S of block j+1 once the
-//                 tile's softmax has read S(j), then P V of block j once P(j) is written
+//   warps 9 / 10  issue tile 0's / tile 1's MMAs: S of block j+1 once the tile's softmax has
+//                 read S(j), then P V of block j once P(j) is written
 //   warps 0-3 / 4-7  softmax of tile 0 / 1, one query row (TMEM lane) per thread: load S,
 //                 release it, running max in the log2 domain and running row sum in
 //                 registers, P = exp2(s - m) as fp16 in registers, then into P_X once the
-//                 previous P V has read it. The two tiles' warps on one SMSP alternate on the
-//                 exponentials. O_X is rescaled in TMEM (load, multiply, store) only when a row's max
+//                 previous P V has read it. The two tiles alternate on the exponentials (named
+//                 barriers: a warp in them polls nothing). O_X is rescaled in TMEM (load, multiply, store) only when a row's max
 //                 grows by more than 2^8, so P stays <= 256 and the rescale is rare.
 #include "fd_internal.h"
 #include "fd_ptx.cuh"
@@ -61,12 +61,12 @@ constexpr int kBarQFull = 0,                 // [buffer] Q tiles of a segment la
               kBarPv = kBarP + 2,              // [tile] P V of block J completed
               kBarOFree = kBarPv + 2,          // [tile] O_X of a segment read by the softmax
               kBarDone = kBarOFree + 2,        // [tile] every MMA of the tile's issuer completed
-              kBarTurn = kBarDone + 2,  // [tile][quarter] the other tile's warp of this SMSP
-                                        // has finished its exponentials: this tile's turn
-              kBarPartDone = kBarTurn + 8,  // [slot] the 8 softmax warps wrote the partial
+              kBarPartDone = kBarDone + 2,  // [slot] the 8 softmax warps wrote the partial
                                             // result of the CTA's first (0) / last (1) segment
               kBarDecided = kBarPartDone + 2,  // the TMA thread has counted both partials
               kNumBars = kBarDecided + 1;
+// named barriers of the turns: tile x's warps wait in kTurn + x for the other tile's
+constexpr int kTurn = 1;
 static_assert(kNumBars * 8 + 8 <= 512, "barrier area");
 static_assert(kSmem <= 227 * 1024, "shared memory");
 // partial results of one (CTA, slot, tile): O as [16][128 rows] float4, then (m, l) per row
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
 #define COUNTERS (kBatched ? bs.cnt : p.counters)
 #define Q_ROW0 (kBatched ? bs.q_row0 : 0)
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_index();
   const int lane = threadIdx.x & 31;
   const uint32_t base = smem_u32(smem);
   const bool aligned = (base & 1023u) == 0;
@@ -198,13 +198,12 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
     }
     for (int x = 0; x < 2; ++x) {
       mbar_init(bar(kBarS + x), 1);
-      mbar_init(bar(kBarSFree + x), 128);
-      mbar_init(bar(kBarP + x), 128);
+      mbar_init(bar(kBarSFree + x), 4);
+      mbar_init(bar(kBarP + x), 4);
       mbar_init(bar(kBarPv + x), 1);
-      mbar_init(bar(kBarOFree + x), 128);
+      mbar_init(bar(kBarOFree + x), 4);
       mbar_init(bar(kBarDone + x), 1);
     }
-    for (int i = 0; i < 8; ++i) mbar_init(bar(kBarTurn + i), 1);
     mbar_init(bar(kBarPartDone), 8);
     mbar_init(bar(kBarPartDone + 1), 8);
     mbar_init(bar(kBarDecided), 1);
@@ -215,6 +214,7 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
   if (STEP_DEV != nullptr) {
     const int t = *STEP_DEV;
     n_keys = (t + 1 < p.window ? t + 1 : p.window) * p.rows_per_chunk;
+    n_keys = __shfl_sync(0xffffffffu, n_keys, 0);  // a warp-uniform value to the compiler
   }
   const int nblk = (n_keys + 127) / 128;
   const WorkRange wr{p.groups * pairs_per_group * nblk, static_cast<int>(gridDim.x)};
@@ -227,25 +227,29 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (warp == 8) {
     // ------------------------------------------------------------ TMA loads
-    if (lane == 0 && aligned && len > 0) {
-      prefetch_tmap(&tmQ);
-      prefetch_tmap(&tmQ8);
-      prefetch_tmap(mK);
-      prefetch_tmap(mV);
+    // (the whole warp runs the loop; one elected lane issues, lane 0 counts the partials)
+    if (aligned && len > 0) {
+      if (elect_one()) {
+        prefetch_tmap(&tmQ);
+        prefetch_tmap(&tmQ8);
+        prefetch_tmap(mK);
+        prefetch_tmap(mV);
+      }
       // Count this CTA's partial results once the softmax warps have stored them. The stores
-      // reach this thread through the barrier (CTA scope); the gpu-scope fence before the
+      // reach lane 0 through the barrier (CTA scope); the gpu-scope fence before the
       // counter update publishes them all (fences are cumulative). The CTA that stores a
       // pair's last part combines the pair. Slot 0 is polled between loads, so that a CTA
       // that finished its first segment early does not end up combining that pair too.
       const PartialSlots ps(wr, u0, len, nblk);
       bool counted[2] = {!ps.has[0], !ps.has[1]};
-      decision[0] = decision[1] = 0;
+      if (lane == 0) decision[0] = decision[1] = 0;
       auto count_slot = [&](int sl) {
         counted[sl] = true;
+        if (lane != 0) return;
         const int pr = ps.pair[sl];
         int owners = 0;  // CTAs holding a part of the pair
         for (int c = wr.cta_of(pr * nblk); c <= wr.cta_of(pr * nblk + nblk - 1); ++c)
@@ -263,18 +267,21 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
       int J = 0;
       bool ok = true;
       for (; J < len && ok; ++J) {
-        if (!counted[0] && mbar_test_wait(bar(kBarPartDone), 0)) count_slot(0);
+        if (!counted[0] && __all_sync(0xffffffffu, mbar_test_wait(bar(kBarPartDone), 0))) {
+          count_slot(0);
+          __syncwarp();
+        }
         const int g = cur.pair / pairs_per_group;
         if (cur.first) {
           // Q of the segment's pair into buffer seg & 1, once the segment two back has done
           // its S MMAs
           const int qb = cur.seg & 1;
-          if (cur.seg >= 2 &&
-              !mbar_wait(bar(kBarQFree + qb), ((cur.seg >> 1) - 1) & 1, ERR_WORD, ERR_WAIT_MMA)) {
+          if (cur.seg >= 2 && !mbar_wait_warp(bar(kBarQFree + qb), ((cur.seg >> 1) - 1) & 1,
+                                              ERR_WORD, ERR_WAIT_MMA)) {
             ok = false;
             break;
           }
-          mbar_expect_tx(bar(kBarQFull + qb), 2 * kQBytes);
+          if (elect_one()) mbar_expect_tx(bar(kBarQFull + qb), 2 * kQBytes);
           // A tile inside one head's rows is one 128-row box (rows past Lq read the fill
           // value); a tile across two heads is loaded in boxes of 8 rows (one 1024-byte
           // swizzle atom each, same shared-memory layout). Rows past the group's last head
@@ -286,51 +293,57 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
             const uint32_t dst = base + kOffQ + (2 * qb + x) * kQBytes;
             const uint32_t qbar = bar(kBarQFull + qb);
             if (hl0 >= hpg) {
-              tma_load_2d(dst, &tmQ, qbar, g * hpg * kHeadDim, Q_ROW0);
+              if (elect_one()) tma_load_2d(dst, &tmQ, qbar, g * hpg * kHeadDim, Q_ROW0);
             } else if (hl1 == hl0 || hl1 >= hpg) {
-              tma_load_2d(dst, &tmQ, qbar, (g * hpg + hl0) * kHeadDim,
-                          Q_ROW0 + rho0 - hl0 * p.lq_pad);
+              if (elect_one())
+                tma_load_2d(dst, &tmQ, qbar, (g * hpg + hl0) * kHeadDim,
+                            Q_ROW0 + rho0 - hl0 * p.lq_pad);
             } else {
               for (int b = 0; b < kBM / 8; ++b) {
                 const int rho = rho0 + 8 * b;
                 int hl = rho / p.lq_pad;
                 int r = rho - hl * p.lq_pad;
                 if (hl >= hpg) hl = r = 0;
-                tma_load_2d(dst + b * 1024, &tmQ8, qbar, (g * hpg + hl) * kHeadDim, Q_ROW0 + r);
+                if (elect_one())
+                  tma_load_2d(dst + b * 1024, &tmQ8, qbar, (g * hpg + hl) * kHeadDim, Q_ROW0 + r);
               }
             }
           }
         }
         const int st = J % kStages;
-        if (!mbar_wait(bar(kBarKvEmpty + st), ((J / kStages) & 1) ^ 1, ERR_WORD, ERR_WAIT_MMA)) {
+        if (!mbar_wait_warp(bar(kBarKvEmpty + st), ((J / kStages) & 1) ^ 1, ERR_WORD,
+                            ERR_WAIT_MMA)) {
           ok = false;
           break;
         }
         const uint32_t b = bar(kBarKvFull + st);
-        mbar_expect_tx(b, kKBytes + kVBytes);
-        tma_load_2d(base + kOffK + st * kKBytes, mK, b, 0, g * p.ring_pitch + cur.kb * 128);
-        tma_load_2d(base + kOffV + st * kVBytes, mV, b, cur.kb * 128, g * kHeadDim);
-        tma_load_2d(base + kOffV + st * kVBytes + kVSub, mV, b, cur.kb * 128 + 64,
-                    g * kHeadDim);
+        if (elect_one()) {
+          mbar_expect_tx(b, kKBytes + kVBytes);
+          tma_load_2d(base + kOffK + st * kKBytes, mK, b, 0, g * p.ring_pitch + cur.kb * 128);
+          tma_load_2d(base + kOffV + st * kVBytes, mV, b, cur.kb * 128, g * kHeadDim);
+          tma_load_2d(base + kOffV + st * kVBytes + kVSub, mV, b, cur.kb * 128 + 64,
+                      g * kHeadDim);
+        }
         if (J + 1 < len) cur.next(len - J - 2, nblk);
       }
       // nothing may be in flight when the CTA exits: the last two Q loads, the last KV loads
       const int nseg = cur.seg + 1;
       for (int sg = nseg - 1; sg >= 0 && sg >= nseg - 2; --sg)
-        mbar_wait(bar(kBarQFull + (sg & 1)), (sg >> 1) & 1, ERR_WORD, ERR_WAIT_TMA);
+        mbar_wait_warp(bar(kBarQFull + (sg & 1)), (sg >> 1) & 1, ERR_WORD, ERR_WAIT_TMA);
       for (int i = J - 1; i >= 0 && i >= J - kStages; --i)
-        mbar_wait(bar(kBarKvFull + i % kStages), (i / kStages) & 1, ERR_WORD, ERR_WAIT_TMA);
+        mbar_wait_warp(bar(kBarKvFull + i % kStages), (i / kStages) & 1, ERR_WORD, ERR_WAIT_TMA);
       for (int sl = 0; sl < 2; ++sl)
-        if (!counted[sl] && mbar_wait(bar(kBarPartDone + sl), 0, ERR_WORD, ERR_WAIT_EPI))
+        if (!counted[sl] && mbar_wait_warp(bar(kBarPartDone + sl), 0, ERR_WORD, ERR_WAIT_EPI))
           count_slot(sl);
-      mbar_arrive(bar(kBarDecided));
+      if (lane == 0) mbar_arrive(bar(kBarDecided));
     }
   } else if (warp == 9 || warp == 10) {
     // ------------------------------------------------------------ MMA issue for tile x
-    // One issuing thread per tile, so neither tile's MMAs wait behind the other's events;
-    // tcgen05.commit tracks only the MMAs of the thread that issues it.
+    // One issuing warp per tile, so neither tile's MMAs wait behind the other's events; the whole
+    // warp runs the loop and its elected lane issues (tcgen05.commit tracks only the MMAs of the
+    // thread that issues it).
     const int x = warp - 9;
-    if (lane == 0 && aligned && len > 0) {
+    if (aligned && len > 0) {
       const uint32_t idesc_s = idesc_bf16_f32(128, 128);
       const uint32_t idesc_o = idesc_f16_f32(128, 64);  // P and V^T are fp16
       // descriptors of the stage bases; K steps of 16 elements add 32 B (2 in the encoded
@@ -344,16 +357,18 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
       // S_X(J) = Q_X K_J^T; after the last block of a segment, release its Q buffer
       auto issue_s = [&](int J, const Cursor& c) -> bool {
         const int qb = c.seg & 1;
-        if (c.first && !mbar_wait(bar(kBarQFull + qb), (c.seg >> 1) & 1, ERR_WORD, ERR_WAIT_TMA))
+        if (c.first && !mbar_wait_warp(bar(kBarQFull + qb), (c.seg >> 1) & 1, ERR_WORD, ERR_WAIT_TMA))
           return false;
-        if (!mbar_wait(bar(kBarKvFull + J % kStages), (J / kStages) & 1, ERR_WORD, ERR_WAIT_TMA))
+        if (!mbar_wait_warp(bar(kBarKvFull + J % kStages), (J / kStages) & 1, ERR_WORD, ERR_WAIT_TMA))
           return false;
         tc_fence_after();
         const uint64_t dq = dq0 + static_cast<uint64_t>((2 * qb * kQBytes) >> 4);
         const uint64_t dk = dk0 + static_cast<uint64_t>(((J % kStages) * kKBytes) >> 4);
-        mma4_bf16_ss(s_tmem, dq, dk, idesc_s, 0u);
-        mma_commit(bar(kBarS + x));
-        if (c.last) mma_commit(bar(kBarQFree + qb));
+        if (elect_one()) {
+          mma4_bf16_ss(s_tmem, dq, dk, idesc_s, 0u);
+          mma_commit(bar(kBarS + x));
+          if (c.last) mma_commit(bar(kBarQFree + qb));
+        }
         return true;
       };
       Cursor cur;
@@ -365,25 +380,27 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
         // S of the next block as soon as the softmax has read S(J)
         if (J + 1 < len) {
           cur.next(len - J - 2, nblk);
-          ok = mbar_wait(bar(kBarSFree + x), J & 1, ERR_WORD, ERR_WAIT_EPI) && issue_s(J + 1, cur);
+          ok = mbar_wait_warp(bar(kBarSFree + x), J & 1, ERR_WORD, ERR_WAIT_EPI) && issue_s(J + 1, cur);
           if (!ok) break;
         }
         // P V of this block once P(J) is written; the first block of a segment overwrites O,
         // so it also waits until the softmax has read the previous segment's O
-        ok = mbar_wait(bar(kBarP + x), J & 1, ERR_WORD, ERR_WAIT_EPI);
+        ok = mbar_wait_warp(bar(kBarP + x), J & 1, ERR_WORD, ERR_WAIT_EPI);
         if (ok && here.first && here.seg > 0)
-          ok = mbar_wait(bar(kBarOFree + x), (here.seg - 1) & 1, ERR_WORD, ERR_WAIT_EPI);
+          ok = mbar_wait_warp(bar(kBarOFree + x), (here.seg - 1) & 1, ERR_WORD, ERR_WAIT_EPI);
         tc_fence_after();
         if (!ok) break;
         const uint64_t dv = dv0 + static_cast<uint64_t>((st * kVBytes) >> 4);
         // keys 0-63 of the block (P columns 0-31, V^T sub-block 0), then keys 64-127
-        mma4_bf16_ts(o_tmem, p_tmem, dv, idesc_o, here.first ? 0u : 1u);
-        mma4_bf16_ts(o_tmem, p_tmem + 32u, dv + static_cast<uint64_t>(kVSub >> 4), idesc_o, 1u);
-        mma_commit(bar(kBarPv + x));
-        mma_commit(bar(kBarKvEmpty + st));  // one of the two arrivals that free the stage
+        if (elect_one()) {
+          mma4_bf16_ts(o_tmem, p_tmem, dv, idesc_o, here.first ? 0u : 1u);
+          mma4_bf16_ts(o_tmem, p_tmem + 32u, dv + static_cast<uint64_t>(kVSub >> 4), idesc_o, 1u);
+          mma_commit(bar(kBarPv + x));
+          mma_commit(bar(kBarKvEmpty + st));  // one of the two arrivals that free the stage
+        }
       }
-      mma_commit(bar(kBarDone + x));
-      mbar_wait(bar(kBarDone + x), 0, ERR_WORD, ERR_WAIT_MMA);
+      if (elect_one()) mma_commit(bar(kBarDone + x));
+      mbar_wait_warp(bar(kBarDone + x), 0, ERR_WORD, ERR_WAIT_MMA);
     }
   } else {
     // ------------------------------------------------------------ softmax, tile x
@@ -397,6 +414,22 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
     const float sl2 = p.scale_log2;
     float m_used = -INFINITY, l_run = 0.f;
     bool ok = aligned;
+    // Turns on the exponentials: tile 0 block J, tile 1 block J, tile 0 block J + 1, ... Each
+    // tile's four warps take theirs together (its P is complete, and its next S free to start,
+    // only when all four are done).
+    auto take_turn = [&](int J) {
+      if (x == 1 || J > 0) named_barrier(kTurn + x, 256);
+    };
+    auto pass_turn = [&](int J) {
+      if (x == 0 || J + 1 < len) named_barrier_arrive(kTurn + 1 - x, 256);
+    };
+    // a warp that gives up still takes and passes the turns from block J on: no one waits for it
+    auto finish_turns = [&](int J) {
+      for (; J < len; ++J) {
+        take_turn(J);
+        pass_turn(J);
+      }
+    };
     Cursor cur;
     cur.begin(u0, len, nblk);
     for (int J = 0; J < len && ok; ++J) {
@@ -405,8 +438,8 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
         m_used = -INFINITY;
         l_run = 0.f;
       }
-      const bool got = mbar_wait(bar(kBarS + x), J & 1, ERR_WORD, ERR_WAIT_MMA);
-      if (!__all_sync(0xffffffffu, got)) {
+      if (!mbar_wait_warp(bar(kBarS + x), J & 1, ERR_WORD, ERR_WAIT_MMA)) {
+        finish_turns(J);
         ok = false;
         break;
       }
@@ -416,7 +449,8 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
       for (int c = 0; c < 4; ++c) tmem_ld_32x32b_x32(s_col + 32 * c, sr[c]);
       tmem_ld_wait();
       tc_fence_before();
-      mbar_arrive(bar(kBarSFree + x));  // S_X may now receive the next block's scores
+      __syncwarp();
+      if (elect_one()) mbar_arrive(bar(kBarSFree + x));  // S_X may receive the next scores
       const int valid = n_keys - cur.kb * 128;
       if (valid < 128) {  // ragged last key block (warp-uniform branch)
 #pragma unroll
@@ -445,46 +479,37 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
       // packed ex2 per two keys; the row sum is a pairwise fp16x2 tree per 64 keys (sums stay
       // below 2^15 because P <= 2^8) added into fp32. This runs while the tensor core may
       // still be reading P_X(J-1): only the store of P(J) and the rescale of O wait for it.
-      // Warp q of tile 0 and warp q of tile 1 share one SMSP; they take turns on the
-      // exponentials (tile 0 block J, tile 1 block J, tile 0 block J+1, ...), so each one's S
-      // load, P V wait and P store run while the other computes.
-      if (x == 1 || J > 0) {
-        const bool turn = mbar_wait(bar(kBarTurn + 4 * x + quarter), (x == 1 ? J : J - 1) & 1,
-                                    ERR_WORD, ERR_WAIT_EPI);
-        if (!__all_sync(0xffffffffu, turn)) {
-          ok = false;
-          break;
-        }
-      }
+      // The tiles take turns, so each one's S load, P V wait and P store run while the other
+      // computes. The sums stay inside the turn: outside it they lengthen the block's chain
+      // (refinement launch 588 -> 638 us).
+      take_turn(J);
       const uint64_t sc2 = pack_f32x2(sl2, sl2);
       const uint64_t ng2 = pack_f32x2(-m_new, -m_new);
       float lsum = 0.f;
-      uint32_t pk[2][32];
+      uint32_t pk[4][16];  // blocks of 16 registers: stores of 32 cost a move per register
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
 #pragma unroll
-        for (int cc = 0; cc < 2; ++cc)
-#pragma unroll
-          for (int e = 0; e < 32; e += 2)
-            pk[half][cc * 16 + (e >> 1)] =
-                exp2_pair_f16(__uint_as_float(sr[2 * half + cc][e]),
-                              __uint_as_float(sr[2 * half + cc][e + 1]), sc2, ng2);
+        for (int e = 0; e < 32; ++e)
+          pk[2 * half + (e >> 4)][e & 15] =
+              exp2_pair_f16(__uint_as_float(sr[2 * half + (e >> 4)][2 * e & 31]),
+                            __uint_as_float(sr[2 * half + (e >> 4)][(2 * e + 1) & 31]), sc2, ng2);
         uint32_t t16[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) t16[i] = hadd2(pk[half][2 * i], pk[half][2 * i + 1]);
+        for (int i = 0; i < 16; ++i)
+          t16[i] = hadd2(pk[2 * half + (i >> 3)][2 * i & 15], pk[2 * half + (i >> 3)][(2 * i + 1) & 15]);
 #pragma unroll
         for (int stride = 8; stride > 0; stride >>= 1)
 #pragma unroll
           for (int i = 0; i < stride; ++i) t16[i] = hadd2(t16[i], t16[i + stride]);
         lsum += f16x2_sum(t16[0]);
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(kBarTurn + 4 * (1 - x) + quarter));
+      pass_turn(J);
       // P_X and O_X are free once the P V of the previous block has completed (for the
       // first block of a segment the previous segment's output already waited for it)
       if (!cur.first) {
-        const bool pv = mbar_wait(bar(kBarPv + x), (J - 1) & 1, ERR_WORD, ERR_WAIT_MMA);
-        if (!__all_sync(0xffffffffu, pv)) {
+        if (!mbar_wait_warp(bar(kBarPv + x), (J - 1) & 1, ERR_WORD, ERR_WAIT_MMA)) {
+          finish_turns(J + 1);
           ok = false;
           break;
         }
@@ -505,17 +530,18 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
         }
       }
       m_used = m_new;
-      tmem_st_32x32b_x32(p_col, pk[0]);
-      tmem_st_32x32b_x32(p_col + 32, pk[1]);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) tmem_st_32x32b_x16(p_col + 16 * c, pk[c]);
       l_run += lsum;
       tmem_st_wait();
       tc_fence_before();
-      mbar_arrive(bar(kBarP + x));
+      __syncwarp();
+      if (elect_one()) mbar_arrive(bar(kBarP + x));
       if (!cur.last) continue;
 
       // -------------------------------------------------------- output of the segment
-      const bool done = mbar_wait(bar(kBarPv + x), J & 1, ERR_WORD, ERR_WAIT_MMA);
-      if (!__all_sync(0xffffffffu, done)) {
+      if (!mbar_wait_warp(bar(kBarPv + x), J & 1, ERR_WORD, ERR_WAIT_MMA)) {
+        finish_turns(J + 1);
         ok = false;
         break;
       }
@@ -533,7 +559,8 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
         }
       }
       tc_fence_before();
-      mbar_arrive(bar(kBarOFree + x));  // O_X may take the next segment's first P V
+      __syncwarp();
+      if (elect_one()) mbar_arrive(bar(kBarOFree + x));  // O_X may take the next segment's P V
       const int g = cur.pair / pairs_per_group;
       const int rho = (2 * (cur.pair - g * pairs_per_group) + x) * kBM + row;
       const int hl = rho / p.lq_pad;
