@@ -65,8 +65,8 @@ constexpr int kBarQFull = 0,                 // [buffer] Q tiles of a segment la
                                             // result of the CTA's first (0) / last (1) segment
               kBarDecided = kBarPartDone + 2,  // the TMA thread has counted both partials
               kNumBars = kBarDecided + 1;
-// named barriers of the turns: tile x's warps wait in kTurn + x for the other tile's
-constexpr int kTurn = 1;
+// named barriers: tile x's warps wait for their turn in kTurn + x; set-up done
+constexpr int kTurn = 1, kReady = 3;
 static_assert(kNumBars * 8 + 8 <= 512, "barrier area");
 static_assert(kSmem <= 227 * 1024, "shared memory");
 // partial results of one (CTA, slot, tile): O as [16][128 rows] float4, then (m, l) per row
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
   const int hpg = p.heads / p.groups;
   const int pairs_per_group = (attention_tiles_per_group(p.Lq, p.heads, p.groups) + 1) / 2;
 
-  if (threadIdx.x == 0) {
+  if (warp == 8 && elect_one()) {
     if (!aligned) atomicOr(ERR_WORD, ERR_SMEM_ALIGN);
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar(kBarQFull + b), 1);
@@ -224,8 +224,12 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
     tmem_alloc(smem_u32(tmem_slot), kTmemCols);
     tmem_relinquish();
   }
+  // the TMA warp needs no TMEM: it goes on to its loads while the others wait for the allocation
+  // (and for the barriers, which it has initialised)
   tc_fence_before();
-  __syncthreads();
+  __syncwarp();
+  if (warp == 8) named_barrier_arrive(kReady, kThreads);
+  else named_barrier(kReady, kThreads);
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 

@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
                       ? (nk < C::kStages ? nk : C::kStages)
                       : 0;
   if (warp == 0) {
-    __syncwarp();
+    __syncwarp();  // thread 0's barriers
     const int nb0 = (cta0 % n_tiles) * BN + static_cast<int>(rank) * C::kBRows;
     for (int kb = 0; kb < pre; ++kb) {
       if (elect_one()) {
@@ -242,6 +242,9 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
     }
   }
   grid_dep_wait();  // inputs written by the previous kernel; TMEM freed by its CTAs
+  // The producer needs no TMEM: it goes on to its loads while the others wait for the allocation
+  // (and for the barriers, which it has initialised).
+  constexpr int kReady = 1;
   if (warp == 1) {
     if (PAIR) {
       tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
@@ -252,9 +255,11 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
     }
   }
   tc_fence_before();
-  __syncthreads();
+  __syncwarp();
+  if (warp == 0) named_barrier_arrive(kReady, C::kThreads);
+  else named_barrier(kReady, C::kThreads);
   tc_fence_after();
-  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // (not used by warp 0)
 
   if (aligned && warp == 0) {
     // ------------------------------------------------------------ TMA producer
