@@ -709,6 +709,7 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
         // head layer 2 with the pixel shuffle (Sec. 3.4 Step 3): each 32-column chunk of the
         // token's row is 32 / rs pixel rows of rs pixels, written as groups of 4 pixels
         const PixelEpi& px = p.pix;
+        if (tile == 0 && warp == 2 && lane == 0 && px.step != nullptr) *px.step += 1;
         const int tau = row / px.tokens, l = row - tau * px.tokens;
         const bool out_row = row_ok && tau < px.frames;
         const int gy = l / px.gw, gx = l - gy * px.gw;

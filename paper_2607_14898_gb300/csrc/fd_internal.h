@@ -68,6 +68,7 @@ struct PixelEpi {
   int frames;       // frames written (rows tau L + l with tau >= frames are dropped)
   int tokens;       // L: rows per frame
   int gh, gw, rs;   // token grid and the spatial upscale (rs % 4 == 0, 32 % rs == 0)
+  int* step;        // chunk counter that the launch advances by one, or null
 };
 
 // One stream of a batched QKV launch: its cache ring, chunk counter and temporal RoPE table.
@@ -258,21 +259,37 @@ cudaError_t launch_rmsnorm(const float* h, const float* g, int M, int D, float e
 // u[r][c] = e4m3(rmsnorm(h)[r][c] * oscale)  (FP8 MLP input)
 cudaError_t launch_rmsnorm_e4m3(const float* h, const float* g, int M, int D, float eps,
                                 uint8_t* u, float oscale, cudaStream_t s);
+// streams of one launch of a chunk's first / last kernel
+constexpr int kMaxStreams = 64;
+struct StartStreams {
+  const float* z[kMaxStreams];   // latent
+  const int* step[kMaxStreams];  // chunk index t on the device
+  float2* rope[kMaxStreams];     // temporal RoPE tables to write
+};
+struct PixelStreams {
+  const float* F[kMaxStreams];
+  void* pix[kMaxStreams];
+  int* step[kMaxStreams];        // chunk counter to advance, or null
+  int frames[kMaxStreams];
+};
 // frame_rows: F rows per refined frame (0 = gh gw, the tokens of a frame)
-cudaError_t launch_pixel_head(const float* F, int frames, int gh, int gw, int C, int rs,
-                              int out_u8, void* pix, cudaStream_t s, int frame_rows = 0);
+cudaError_t launch_pixel_head(const PixelStreams& st, int n, int gh, int gw, int C, int rs,
+                              int out_u8, cudaStream_t s, int frame_rows = 0);
 cudaError_t launch_kv_append(const float* k, const float* v, int groups, int rows, int slot,
                              int ring_pitch, __nv_bfloat16* k_ring, __half* vt_ring,
                              cudaStream_t s);
-cudaError_t launch_advance(int* step_dev, cudaStream_t s);
 // failure-path check: a bounded wait that runs out after limit_ns and records ERR_WAIT_CHECK
 cudaError_t launch_wait_check(int* err, unsigned long long limit_ns, cudaStream_t s);
-// Temporal RoPE table of one chunk: for each block of `frames[k]` frames per chunk (k < nsets),
+// Temporal RoPE table of chunk t: for each block of `frames[k]` frames per chunk (k < nsets),
 // entries [off_k + tau][i] = (cos, sin)((t * frames[k] + tau) * inv_freq[i]), i < band_t,
-// computed in fp64 (t read from step_dev, or t_host when step_dev is null).
-cudaError_t launch_rope_table(const int* step_dev, int t_host, int nsets, const int* frames,
-                              int band_t, const double* inv_freq, float2* table,
-                              cudaStream_t s);
+// computed in fp64.
+cudaError_t launch_rope_table(int t, int nsets, const int* frames, int band_t,
+                              const double* inv_freq, float2* table, cudaStream_t s);
+// A chunk's first launch: the tables of each stream's chunk (t read from its step) and the
+// PixelUnshuffle of its latent into x0 + i x0_stride
+cudaError_t launch_chunk_start(const StartStreams& st, int n, int C, int H, int W, int p,
+                               __nv_bfloat16* x0, size_t x0_stride, int nsets, const int* frames,
+                               int band_t, const double* inv_freq, cudaStream_t s);
 constexpr int kMaxRopeSets = 2;
 
 // ---- hooks of the training step (fd_train.cu) into the runtime (flashdec.cu)

@@ -6,7 +6,9 @@
 //   pixel_head   F fp32 [frames*L][C r_s^2] -> PixelShuffle(r_s) + clamp to [-1, 1], fp32 or
 //                uint8 (Sec. 3.4 "Step 3"); one thread per 4 consecutive output pixels
 //   kv_append    fp32 K, V of one chunk -> ring slot (K rows bf16, V transposed fp16) (Sec. 3.3)
-//   advance      chunk counter t += 1 (device-resident, so a captured graph can be replayed)
+//                and, in the decode, chunk counter t += 1 (device-resident, so a captured graph
+//                can be replayed)
+//   chunk_start  a chunk's unshuffle and its temporal RoPE tables in one launch
 //   wait_check   failure-path check: a wait on an mbarrier that nothing arrives at, through
 //                the decode kernels' bounded wait, gives up after a short limit and returns
 #include "fd_internal.h"
@@ -14,21 +16,26 @@
 
 namespace fd {
 
-__global__ void unshuffle_kernel(const float* __restrict__ z, int C, int H, int W, int p,
-                                 __nv_bfloat16* __restrict__ x0) {
-  grid_dep_wait();
-  grid_dep_launch();
+// blocks 0 .. blocks - 1 of the grid's x
+__device__ __forceinline__ void unshuffle(const float* __restrict__ z, int C, int H, int W, int p,
+                                          __nv_bfloat16* __restrict__ x0, int blocks) {
   const int gw = W / p;
   const int cin = C * p * p;
   const int total = (H / p) * gw * cin;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += gridDim.x * blockDim.x) {
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += blocks * blockDim.x) {
     const int l = idx / cin, ch = idx - l * cin;
     const int c = ch / (p * p), ij = ch - c * p * p;
     const int i = ij / p, j = ij - i * p;
     const int h = l / gw, w = l - h * gw;
     x0[idx] = __float2bfloat16_rn(z[(static_cast<size_t>(c) * H + h * p + i) * W + w * p + j]);
   }
+}
+
+__global__ void unshuffle_kernel(const float* __restrict__ z, int C, int H, int W, int p,
+                                 __nv_bfloat16* __restrict__ x0) {
+  grid_dep_wait();
+  grid_dep_launch();
+  unshuffle(z, C, H, W, p, x0, gridDim.x);
 }
 
 // one warp per row, the row held in registers (D / 128 float4 per lane for D / 128 in
@@ -108,11 +115,17 @@ __global__ void rmsnorm_kernel(const float* __restrict__ h, const float* __restr
 
 
 // pix[c][tau][y][x] = clamp(F[tau*L + (y/rs)*gw + x/rs][c*rs*rs + (y%rs)*rs + x%rs]); rs % 4 == 0
-// frame tau's tokens are rows tau * frame_rows .. + gh gw - 1 of F (frame_rows >= gh gw)
-__global__ void pixel_head_kernel(const float* __restrict__ F, int frames, int frame_rows, int gh,
-                                  int gw, int C, int rs, int out_u8, void* __restrict__ pix) {
+// frame tau's tokens are rows tau * frame_rows .. + gh gw - 1 of F (frame_rows >= gh gw). Grid y:
+// stream (its F, pixels and frame count; its chunk counter, if any, advances by one).
+__global__ void pixel_head_kernel(const __grid_constant__ PixelStreams st, int frame_rows, int gh,
+                                  int gw, int C, int rs, int out_u8) {
   grid_dep_wait();
   grid_dep_launch();
+  const float* __restrict__ F = st.F[blockIdx.y];
+  void* __restrict__ pix = st.pix[blockIdx.y];
+  const int frames = st.frames[blockIdx.y];
+  if (blockIdx.x == 0 && threadIdx.x == 0 && st.step[blockIdx.y] != nullptr)
+    *st.step[blockIdx.y] += 1;
   const int Wo = gw * rs, Ho = gh * rs;
   const int ld = C * rs * rs;
   const int q_per_row = Wo / 4;
@@ -172,23 +185,15 @@ __global__ void kv_append_kernel(const float* __restrict__ k, const float* __res
   }
 }
 
-__global__ void advance_kernel(int* step) {
-  grid_dep_wait();
-  grid_dep_launch();
-  *step += 1;
-}
-
 struct RopeSets {
   int frames[kMaxRopeSets];
   double inv_freq[kRopePairs];
 };
 
-// one thread per (set, frame, pair): angles reduced and evaluated in fp64, stored as fp32
-__global__ void rope_table_kernel(const int* step_dev, int t_host, int nsets, int band_t,
-                                  RopeSets sets, float2* table) {
-  grid_dep_wait();
-  grid_dep_launch();
-  const int t = step_dev ? *step_dev : t_host;
+// one thread per (set, frame, pair) of one block: angles reduced and evaluated in fp64, stored as
+// fp32
+__device__ __forceinline__ void rope_table(int t, int nsets, int band_t, const RopeSets& sets,
+                                           float2* table) {
   int off = 0;
   for (int k = 0; k < nsets; ++k) {
     const int n = sets.frames[k] * band_t;
@@ -201,6 +206,27 @@ __global__ void rope_table_kernel(const int* step_dev, int t_host, int nsets, in
     }
     off += n;
   }
+}
+__global__ void rope_table_kernel(int t, int nsets, int band_t,
+                                  const __grid_constant__ RopeSets sets, float2* table) {
+  grid_dep_wait();
+  grid_dep_launch();
+  rope_table(t, nsets, band_t, sets, table);
+}
+
+// A chunk's first launch: the PixelUnshuffle of each stream's latent (grid y = stream) and, in each
+// stream's last block, its temporal RoPE tables. One launch where two per stream cost ~2.5 us each
+// under dependent launch, more than their work (0.6 MB and some 60 sines).
+__global__ void chunk_start_kernel(const __grid_constant__ StartStreams st, int C, int H, int W,
+                                   int p, __nv_bfloat16* x0, size_t x0_stride, int nsets,
+                                   int band_t, const __grid_constant__ RopeSets sets) {
+  grid_dep_wait();
+  grid_dep_launch();
+  const int i = blockIdx.y, last = gridDim.x - 1;
+  if (blockIdx.x == static_cast<unsigned>(last))
+    rope_table(*st.step[i], nsets, band_t, sets, st.rope[i]);
+  else
+    unshuffle(st.z[i], C, H, W, p, x0 + i * x0_stride, last);
 }
 
 static int grid_for(long long work, int threads) {
@@ -228,12 +254,14 @@ cudaError_t launch_rmsnorm_e4m3(const float* h, const float* g, int M, int D, fl
                     static_cast<void*>(u), oscale);
 }
 
-cudaError_t launch_pixel_head(const float* F, int frames, int gh, int gw, int C, int rs,
-                              int out_u8, void* pix, cudaStream_t s, int frame_rows) {
+cudaError_t launch_pixel_head(const PixelStreams& st, int n, int gh, int gw, int C, int rs,
+                              int out_u8, cudaStream_t s, int frame_rows) {
+  int frames = 0;
+  for (int i = 0; i < n; ++i) frames = st.frames[i] > frames ? st.frames[i] : frames;
   const long long total = static_cast<long long>(C) * frames * gh * rs * gw * rs / 4;
   if (frame_rows == 0) frame_rows = gh * gw;
-  return launch_pdl(pixel_head_kernel, dim3(grid_for(total, 256)), dim3(256), 0, s, F, frames,
-                    frame_rows, gh, gw, C, rs, out_u8, pix);
+  return launch_pdl(pixel_head_kernel, dim3(grid_for(total, 256), n), dim3(256), 0, s, st,
+                    frame_rows, gh, gw, C, rs, out_u8);
 }
 
 cudaError_t launch_kv_append(const float* k, const float* v, int groups, int rows, int slot,
@@ -244,16 +272,32 @@ cudaError_t launch_kv_append(const float* k, const float* v, int groups, int row
                     k_ring, vt_ring);
 }
 
-cudaError_t launch_rope_table(const int* step_dev, int t_host, int nsets, const int* frames,
-                              int band_t, const double* inv_freq, float2* table,
-                              cudaStream_t s) {
+static cudaError_t rope_sets(int nsets, const int* frames, int band_t, const double* inv_freq,
+                             RopeSets& sets) {
   if (nsets < 1 || nsets > kMaxRopeSets || band_t < 1 || band_t > kRopePairs)
     return cudaErrorInvalidValue;
-  RopeSets sets{};
   for (int k = 0; k < nsets; ++k) sets.frames[k] = frames[k];
   for (int i = 0; i < band_t; ++i) sets.inv_freq[i] = inv_freq[i];
-  return launch_pdl(rope_table_kernel, dim3(1), dim3(128), 0, s, step_dev, t_host, nsets, band_t,
-                    sets, table);
+  return cudaSuccess;
+}
+
+cudaError_t launch_rope_table(int t, int nsets, const int* frames, int band_t,
+                              const double* inv_freq, float2* table, cudaStream_t s) {
+  RopeSets sets{};
+  const cudaError_t e = rope_sets(nsets, frames, band_t, inv_freq, sets);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(rope_table_kernel, dim3(1), dim3(128), 0, s, t, nsets, band_t, sets, table);
+}
+
+cudaError_t launch_chunk_start(const StartStreams& st, int n, int C, int H, int W, int p,
+                               __nv_bfloat16* x0, size_t x0_stride, int nsets, const int* frames,
+                               int band_t, const double* inv_freq, cudaStream_t s) {
+  RopeSets sets{};
+  const cudaError_t e = rope_sets(nsets, frames, band_t, inv_freq, sets);
+  if (e != cudaSuccess) return e;
+  const long long total = static_cast<long long>(H / p) * (W / p) * C * p * p;
+  return launch_pdl(chunk_start_kernel, dim3(grid_for(total, 256) + 1, n), dim3(256), 0, s, st, C,
+                    H, W, p, x0, x0_stride, nsets, band_t, sets);
 }
 
 // One thread waits, with the decode kernels' bounded wait (mbar_wait_for) and a limit of
@@ -272,10 +316,6 @@ __global__ void wait_check_kernel(int* err, unsigned long long limit_ns) {
 cudaError_t launch_wait_check(int* err, unsigned long long limit_ns, cudaStream_t s) {
   wait_check_kernel<<<1, 32, 0, s>>>(err, limit_ns);
   return cudaGetLastError();
-}
-
-cudaError_t launch_advance(int* step_dev, cudaStream_t s) {
-  return launch_pdl(advance_kernel, dim3(1), dim3(1), 0, s, step_dev);
 }
 
 }  // namespace fd

@@ -662,17 +662,16 @@ fd_status decode_one(fd_handle h, const float* latent, void* pixels, cudaStream_
     const int frames[2] = {1, d.rt};
     double inv[fd::kRopePairs];
     temporal_inv_freq(h->cfg.rope_base, inv);
-    const int* step = h->state;
-    float2* tab = h->rope_tab;
-    if ((st = traced(h, FD_K_ROPE, s, [&] {
-           return fd::launch_rope_table(step, 0, 2, frames, rope_band_t(), inv, tab, s);
+    fd::StartStreams in{};
+    in.z[0] = latent;
+    in.step[0] = h->state;
+    in.rope[0] = h->rope_tab;
+    if ((st = traced(h, FD_K_UNSHUFFLE, s, [&] {
+           return fd::launch_chunk_start(in, 1, d.C, d.H, d.W, d.p, h->x0, 0, 2, frames,
+                                         rope_band_t(), inv, s);
          })))
       return st;
   }
-  __nv_bfloat16* x0 = h->x0;
-  if ((st = traced(h, FD_K_UNSHUFFLE, s,
-                   [&] { return fd::launch_unshuffle(latent, d.C, d.H, d.W, d.p, x0, s); })))
-    return st;
   fd::GemmParams pe{};
   pe.epi = fd::EPI_F32;
   pe.out_f32 = h->h;
@@ -706,25 +705,24 @@ fd_status decode_one(fd_handle h, const float* latent, void* pixels, cudaStream_
   const int frames = d.f1 && h->t_host == 0 ? 1 : d.rt;
   fd::GemmParams pf{};
   if (fd::gemm_pixel_epilogue_ok(w->head2.bn, w->head2.pair, d.rs)) {
-    // the pixel shuffle, clamp (and uint8 code) in the product's epilogue: F is never stored
+    // the pixel shuffle, clamp (and uint8 code) in the product's epilogue: F is never stored; the
+    // launch also advances the chunk counter
     pf.epi = fd::EPI_PIXEL;
-    pf.pix = {pixels, d.u8 ? 1 : 0, frames, d.L, d.gh, d.gw, d.rs};
-    if ((st = run_linear(h, FD_K_HEAD2, h->tm_hidH, w->head2, R, pf, h->so_F, s))) return st;
-    int* state = h->state;
-    return traced(h, FD_K_ADVANCE, s, [&] { return fd::launch_advance(state, s); });
+    pf.pix = {pixels, d.u8 ? 1 : 0, frames, d.L, d.gh, d.gw, d.rs, h->state};
+    return run_linear(h, FD_K_HEAD2, h->tm_hidH, w->head2, R, pf, h->so_F, s);
   }
   pf.epi = fd::EPI_F32;
   pf.out_f32 = h->F;
   pf.ld_out = d.head_out;
   if ((st = run_linear(h, FD_K_HEAD2, h->tm_hidH, w->head2, R, pf, h->so_F, s))) return st;
-  const float* F = h->F;
-  if ((st = traced(h, FD_K_PIXEL, s, [&] {
-         return fd::launch_pixel_head(F, frames, d.gh, d.gw, d.Cout, d.rs, d.u8 ? 1 : 0, pixels,
-                                      s);
-       })))
-    return st;
-  int* state = h->state;
-  return traced(h, FD_K_ADVANCE, s, [&] { return fd::launch_advance(state, s); });
+  fd::PixelStreams out{};
+  out.F[0] = h->F;
+  out.pix[0] = pixels;
+  out.step[0] = h->state;
+  out.frames[0] = frames;
+  return traced(h, FD_K_PIXEL, s, [&] {
+    return fd::launch_pixel_head(out, 1, d.gh, d.gw, d.Cout, d.rs, d.u8 ? 1 : 0, s);
+  });
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -879,21 +877,20 @@ fd_status decode_batch(fd_batch b, fd_handle* hs, int n, const float* const* lat
   const fd_weights w = b->w;
   fd_handle h0 = hs[0];
   fd_status st;
-  const int bt = rope_band_t();
-  for (int i = 0; i < n; ++i) {
-    const int frames[2] = {1, d.rt};
+  {
+    const int bt = rope_band_t(), frames[2] = {1, d.rt};
     double inv[fd::kRopePairs];
     temporal_inv_freq(h0->cfg.rope_base, inv);
-    const int* step = hs[i]->state;
-    float2* tab = b->rope + static_cast<size_t>(i) * (1 + d.rt) * bt;
-    if ((st = traced(hs[i], FD_K_ROPE, s, [&] {
-           return fd::launch_rope_table(step, 0, 2, frames, bt, inv, tab, s);
+    fd::StartStreams in{};
+    for (int i = 0; i < n; ++i) {
+      in.z[i] = latents[i];
+      in.step[i] = hs[i]->state;
+      in.rope[i] = b->rope + static_cast<size_t>(i) * (1 + d.rt) * bt;
+    }
+    if ((st = traced(h0, FD_K_UNSHUFFLE, s, [&] {
+           return fd::launch_chunk_start(in, n, d.C, d.H, d.W, d.p, b->x0,
+                                         static_cast<size_t>(b->Lp) * d.cin, 2, frames, bt, inv, s);
          })))
-      return st;
-    __nv_bfloat16* x0 = b->x0 + static_cast<size_t>(i) * b->Lp * d.cin;
-    const float* z = latents[i];
-    if ((st = traced(hs[i], FD_K_UNSHUFFLE, s,
-                     [&] { return fd::launch_unshuffle(z, d.C, d.H, d.W, d.p, x0, s); })))
       return st;
   }
   const int MB = n * b->Lp, MR = n * b->Rp;
@@ -942,24 +939,17 @@ fd_status decode_batch(fd_batch b, fd_handle* hs, int n, const float* const* lat
   pf.out_f32 = b->F;
   pf.ld_out = d.head_out;
   if ((st = run_linear(h0, FD_K_HEAD2, b->tm_hidH, b->head2, MR, pf, b->so_F, s))) return st;
+  fd::PixelStreams out{};
   for (int i = 0; i < n; ++i) {
-    const float* F = b->F + static_cast<size_t>(i) * b->Rp * d.head_out;
-    const int frames = d.f1 && hs[i]->t_host == 0 ? 1 : d.rt;
-    void* pix = pixels[i];
-    const int Lp = b->Lp;
-    if ((st = traced(hs[i], FD_K_PIXEL, s, [&] {
-           return fd::launch_pixel_head(F, frames, d.gh, d.gw, d.Cout, d.rs, d.u8 ? 1 : 0, pix, s,
-                                        Lp);
-         })))
-      return st;
-    int* state = hs[i]->state;
-    if ((st = traced(hs[i], FD_K_ADVANCE, s, [&] { return fd::launch_advance(state, s); })))
-      return st;
+    out.F[i] = b->F + static_cast<size_t>(i) * b->Rp * d.head_out;
+    out.pix[i] = pixels[i];
+    out.step[i] = hs[i]->state;
+    out.frames[i] = d.f1 && hs[i]->t_host == 0 ? 1 : d.rt;
   }
-  return FD_OK;
+  return traced(h0, FD_K_PIXEL, s, [&] {
+    return fd::launch_pixel_head(out, n, d.gh, d.gw, d.Cout, d.rs, d.u8 ? 1 : 0, s, b->Lp);
+  });
 }
-
-
 
 constexpr int kMaxAttnParts = 4096;  // CTAs of one attention launch (fd_op_attention)
 
@@ -2199,7 +2189,7 @@ fd_status fd_op_linear_pixel(int M, int K, const void* A, const void* W, const f
   p.M = M; p.N = static_cast<int>(N); p.K = K; p.epi = fd::EPI_PIXEL; p.bias = bias;
   p.err = err_dev;
   p.pix = {pixels, out_dtype == FD_DTYPE_U8 ? 1 : 0, frames, static_cast<int>(L), grid_h, grid_w,
-           rs};
+           rs, nullptr};
   return launch_ok(fd::launch_gemm(ta, tb, ta, ta, ta, p, 256, false, num_sms(),
                                    static_cast<cudaStream_t>(stream)));
 }
@@ -2405,7 +2395,7 @@ fd_status fd_op_rope_table(int t, int frames_per_chunk, float rope_base, float* 
   double inv[fd::kRopePairs];
   temporal_inv_freq(rope_base, inv);
   const int frames[1] = {frames_per_chunk};
-  return launch_ok(fd::launch_rope_table(nullptr, t, 1, frames, rope_band_t(), inv,
+  return launch_ok(fd::launch_rope_table(t, 1, frames, rope_band_t(), inv,
                                          reinterpret_cast<float2*>(table),
                                          static_cast<cudaStream_t>(stream)));
 }
@@ -2497,8 +2487,12 @@ fd_status fd_op_pixel_head(const float* F, int frames, int grid_h, int grid_w, i
   if (out_dtype != FD_DTYPE_F32 && out_dtype != FD_DTYPE_U8) return FD_ERR_INVALID_ARG;
   fd_status st = check_device();
   if (st) return st;
-  return launch_ok(fd::launch_pixel_head(F, frames, grid_h, grid_w, channels, rs,
-                                         out_dtype == FD_DTYPE_U8 ? 1 : 0, pixels,
+  fd::PixelStreams out{};
+  out.F[0] = F;
+  out.pix[0] = pixels;
+  out.frames[0] = frames;
+  return launch_ok(fd::launch_pixel_head(out, 1, grid_h, grid_w, channels, rs,
+                                         out_dtype == FD_DTYPE_U8 ? 1 : 0,
                                          static_cast<cudaStream_t>(stream)));
 }
 
