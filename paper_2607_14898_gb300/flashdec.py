@@ -176,17 +176,24 @@ def pack_blob(cfg, weights: dict) -> np.ndarray:
 
 def _stream_ptr(stream) -> int:
     if stream is None:
+        # torch.cuda.current_stream().cuda_stream without its Stream object: 0.4 against 3.1 us,
+        # a fifth of a kernel-level call's host time
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return int(getattr(stream, "cuda_stream", stream))
 
 
 def _ptr(x) -> int:
+    # tensors first: a kernel-level call marshals up to a dozen of them
+    try:
+        return x.data_ptr()
+    except AttributeError:
+        pass
     if x is None:
         return 0
     if isinstance(x, np.ndarray):
         return int(x.ctypes.data)
-    return int(x.data_ptr()) if hasattr(x, "data_ptr") else int(x)
+    return int(x)
 
 
 def check_buffer(x, what: str, nbytes: int, dtype: str, on_device: bool,
