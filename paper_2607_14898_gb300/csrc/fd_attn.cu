@@ -28,8 +28,8 @@
 //   warps 0-3 / 4-7  softmax of tile 0 / 1, one query row (TMEM lane) per thread: load S,
 //                 release it, running max in the log2 domain and running row sum in
 //                 registers, P = exp2(s - m) as fp16 in registers, then into P_X once the
-//                 previous P V has read it. The two tiles alternate on the exponentials (named
-//                 barriers: a warp in them polls nothing). O_X is rescaled in TMEM (load, multiply, store) only when a row's max
+//                 previous P V has read it. The two tiles alternate on the exponentials, half a
+//                 block apart (named barriers: a warp in them polls nothing). O_X is rescaled in TMEM (load, multiply, store) only when a row's max
 //                 grows by more than 2^8, so P stays <= 256 and the rescale is rare.
 #include "fd_internal.h"
 #include "fd_ptx.cuh"
@@ -65,8 +65,8 @@ constexpr int kBarQFull = 0,                 // [buffer] Q tiles of a segment la
                                             // result of the CTA's first (0) / last (1) segment
               kBarDecided = kBarPartDone + 2,  // the TMA thread has counted both partials
               kNumBars = kBarDecided + 1;
-// named barriers: tile x's warps wait for their turn in kTurn + x; set-up done
-constexpr int kTurn = 1, kReady = 3;
+// named barriers: set-up done; warp q of tile x waits for its turn in kTurn + 4 x + q
+constexpr int kReady = 1, kTurn = 2;
 static_assert(kNumBars * 8 + 8 <= 512, "barrier area");
 static_assert(kSmem <= 227 * 1024, "shared memory");
 // partial results of one (CTA, slot, tile): O as [16][128 rows] float4, then (m, l) per row
@@ -418,14 +418,14 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
     const float sl2 = p.scale_log2;
     float m_used = -INFINITY, l_run = 0.f;
     bool ok = aligned;
-    // Turns on the exponentials: tile 0 block J, tile 1 block J, tile 0 block J + 1, ... Each
-    // tile's four warps take theirs together (its P is complete, and its next S free to start,
-    // only when all four are done).
+    // Turns on the exponentials: tile 0 block J, tile 1 block J, tile 0 block J + 1, ... Warps q
+    // of the two tiles share a scheduler and take turns with each other only (541 us in the
+    // refinement launch, 544 with all four warps of a tile at one barrier).
     auto take_turn = [&](int J) {
-      if (x == 1 || J > 0) named_barrier(kTurn + x, 256);
+      if (x == 1 || J > 0) named_barrier(kTurn + 4 * x + quarter, 64);
     };
     auto pass_turn = [&](int J) {
-      if (x == 0 || J + 1 < len) named_barrier_arrive(kTurn + 1 - x, 256);
+      if (x == 0 || J + 1 < len) named_barrier_arrive(kTurn + 4 * (1 - x) + quarter, 64);
     };
     // a warp that gives up still takes and passes the turns from block J on: no one waits for it
     auto finish_turns = [&](int J) {
@@ -484,31 +484,37 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
       // below 2^15 because P <= 2^8) added into fp32. This runs while the tensor core may
       // still be reading P_X(J-1): only the store of P(J) and the rescale of O wait for it.
       // The tiles take turns, so each one's S load, P V wait and P store run while the other
-      // computes. The sums stay inside the turn: outside it they lengthen the block's chain
-      // (refinement launch 588 -> 638 us).
+      // computes; the turn passes after half of the exponentials (refinement launch: 572 us after
+      // all of them, 544 after half, 547 / 556 after 3/8 and 5/8, 576 at once, 653 untaken).
       take_turn(J);
       const uint64_t sc2 = pack_f32x2(sl2, sl2);
       const uint64_t ng2 = pack_f32x2(-m_new, -m_new);
       float lsum = 0.f;
       uint32_t pk[4][16];  // blocks of 16 registers: stores of 32 cost a move per register
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
+      auto exps = [&](int half) {
 #pragma unroll
         for (int e = 0; e < 32; ++e)
           pk[2 * half + (e >> 4)][e & 15] =
               exp2_pair_f16(__uint_as_float(sr[2 * half + (e >> 4)][2 * e & 31]),
                             __uint_as_float(sr[2 * half + (e >> 4)][(2 * e + 1) & 31]), sc2, ng2);
+      };
+      auto half_sum = [&](int half) {
         uint32_t t16[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i)
-          t16[i] = hadd2(pk[2 * half + (i >> 3)][2 * i & 15], pk[2 * half + (i >> 3)][(2 * i + 1) & 15]);
+          t16[i] = hadd2(pk[2 * half + (i >> 3)][2 * i & 15],
+                         pk[2 * half + (i >> 3)][(2 * i + 1) & 15]);
 #pragma unroll
         for (int stride = 8; stride > 0; stride >>= 1)
 #pragma unroll
           for (int i = 0; i < stride; ++i) t16[i] = hadd2(t16[i], t16[i + stride]);
         lsum += f16x2_sum(t16[0]);
-      }
+      };
+      exps(0);
       pass_turn(J);
+      half_sum(0);
+      exps(1);
+      half_sum(1);
       // P_X and O_X are free once the P V of the previous block has completed (for the
       // first block of a segment the previous segment's output already waited for it)
       if (!cur.first) {
