@@ -190,10 +190,11 @@ __device__ __forceinline__ uint32_t mapa_rank(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-// arrive (release, cluster scope) on an mbarrier given by its shared::cluster address
+// Arrive on an mbarrier given by its shared::cluster address. It hands over TMEM columns whose reads
+// have completed and no memory, so it carries no cluster-scope release: that fence waits for the
+// thread's outstanding stores, measured at 2200-4000 cycles between two tiles of a CTA pair.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar_cluster) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster)
-               : "memory");
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
 // 2D tile load into this CTA's shared memory that completes on an mbarrier of either CTA of
 // the pair (bar_cluster: shared::cluster address, e.g. the even CTA's)
