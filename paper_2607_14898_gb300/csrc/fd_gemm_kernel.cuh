@@ -89,27 +89,38 @@ __device__ __forceinline__ void put_row_sw64(uint8_t* buf, int row, const uint32
         make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
 }
 
-// 1 + erf(a), after Abramowitz & Stegun, Handbook of Mathematical Functions, formula 7.1.26:
-// for b = |a|, erf(b) = 1 - (a1 t + a2 t^2 + a3 t^3 + a4 t^4 + a5 t^5) e^(-b^2) with
-// t = 1 / (1 + p b), absolute error at most 1.5e-7. With E = the polynomial times e^(-b^2),
-// 1 + erf(a) = 2 - E for a >= 0 and E for a < 0 (erf is odd), so the negative side has no
-// cancellation. In fp32 with the hardware reciprocal and exp2 (a few ulp each) the error stays
-// near 1e-7, far below the bf16 (2^-9) and e4m3 (2^-4) rounding of the GELU outputs.
-__device__ __forceinline__ float one_plus_erf(float a) {
-  const float b = fabsf(a);
-  float t;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f, b, 1.0f)));
-  float y = fmaf(1.061405429f, t, -1.453152027f);
-  y = fmaf(y, t, 1.421413741f);
-  y = fmaf(y, t, -0.284496736f);
-  y = fmaf(y, t, 0.254829592f);
-  const float e = y * t * ex2_approx(-(b * b) * 1.44269504088896341f);  // erfc(b)
-  return a >= 0.f ? 2.0f - e : e;
-}
-
-// GELU, exact (erf) form: x Phi(x) = 0.5 x (1 + erf(x / sqrt 2))
-__device__ __forceinline__ float gelu_erf(float x) {
-  return 0.5f * x * one_plus_erf(x * 0.70710678118654752f);
+// GELU, exact (erf) form, of two values: x Phi(x) = 0.5 x (1 + erf(a)), a = x / sqrt 2. 1 + erf(a)
+// after Abramowitz & Stegun, Handbook of Mathematical Functions, formula 7.1.26: for b = |a|,
+// erf(b) = 1 - (a1 t + a2 t^2 + a3 t^3 + a4 t^4 + a5 t^5) e^(-b^2) with t = 1 / (1 + p b), absolute
+// error at most 1.5e-7. With E = the polynomial times e^(-b^2), 1 + erf(a) = 2 - E for a >= 0 and
+// E for a < 0 (erf is odd), so the negative side has no cancellation. In fp32 with the hardware
+// reciprocal and exp2 (a few ulp each) the error stays near 1e-7, far below the bf16 (2^-9) and
+// e4m3 (2^-4) rounding of the GELU outputs.
+// Packed multiplies and FMAs (each rounded as its scalar form) leave the two MUFU operations per
+// value as the bound: 4096 of the 5300 cycles of a 128 x 256 tile. Against scalar code, 6240 x 4096
+// x 1024: 39.6 -> 37.6 us.
+__device__ __forceinline__ uint64_t gelu_erf_x2(uint64_t x) {
+  auto both = [](float v) { return pack_f32x2(v, v); };
+  const uint64_t a = mul_f32x2(x, both(0.70710678118654752f));
+  float a0, a1, t0, t1, q0, q1;
+  unpack_f32x2(a, a0, a1);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(fmaf(0.3275911f, fabsf(a0), 1.0f)));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(fmaf(0.3275911f, fabsf(a1), 1.0f)));
+  const uint64_t t = pack_f32x2(t0, t1);
+  uint64_t y = fma_f32x2(both(1.061405429f), t, both(-1.453152027f));
+  y = fma_f32x2(y, t, both(1.421413741f));
+  y = fma_f32x2(y, t, both(-0.284496736f));
+  y = fma_f32x2(y, t, both(0.254829592f));
+  const uint64_t q = mul_f32x2(mul_f32x2(a, a), both(-1.44269504088896341f));
+  unpack_f32x2(q, q0, q1);
+  const float p0 = ex2_approx(q0), p1 = ex2_approx(q1);
+  const uint64_t yt = mul_f32x2(y, t);
+  float z0, z1, e0, e1;
+  unpack_f32x2(yt, z0, z1);
+  unpack_f32x2(mul_f32x2(yt, pack_f32x2(p0, p1)), e0, e1);
+  e0 = a0 >= 0.f ? 2.0f - e0 : e0;
+  e1 = a1 >= 0.f ? 2.0f - e1 : e1;
+  return mul_f32x2(mul_f32x2(x, both(0.5f)), pack_f32x2(e0, e1));
 }
 
 // 32 consecutive fp32 values (16-byte aligned) as eight vector loads; the same for every lane
@@ -583,10 +594,14 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
             load32(p.bias + col + 32, b1);
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              w[j] = pack_bf16x2(gelu_erf(__uint_as_float(r0[2 * j]) + b0[2 * j]),
-                                 gelu_erf(__uint_as_float(r0[2 * j + 1]) + b0[2 * j + 1]));
-              w[16 + j] = pack_bf16x2(gelu_erf(__uint_as_float(r1[2 * j]) + b1[2 * j]),
-                                      gelu_erf(__uint_as_float(r1[2 * j + 1]) + b1[2 * j + 1]));
+              auto gelu2 = [](const uint32_t* r, const float* b) {
+                const uint64_t acc2 = pack_f32x2(__uint_as_float(r[0]), __uint_as_float(r[1]));
+                float g0, g1;
+                unpack_f32x2(gelu_erf_x2(add_f32x2(acc2, pack_f32x2(b[0], b[1]))), g0, g1);
+                return pack_bf16x2(g0, g1);
+              };
+              w[j] = gelu2(r0 + 2 * j, b0 + 2 * j);
+              w[16 + j] = gelu2(r1 + 2 * j, b1 + 2 * j);
             }
           }
           uint8_t* buf = acquire();
@@ -618,9 +633,14 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
             for (int j = 0; j < 8; ++j) {
               float f[4];
 #pragma unroll
-              for (int e = 0; e < 4; ++e)
-                f[e] = gelu_erf(fmaf(__uint_as_float(r[4 * j + e]), cs[4 * j + e], bb[4 * j + e])) *
-                       p.out_scale;
+              for (int e = 0; e < 4; e += 2) {
+                const int i = 4 * j + e;
+                const uint64_t x2 = fma_f32x2(
+                    pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])),
+                    pack_f32x2(cs[i], cs[i + 1]), pack_f32x2(bb[i], bb[i + 1]));
+                unpack_f32x2(mul_f32x2(gelu_erf_x2(x2), pack_f32x2(p.out_scale, p.out_scale)), f[e],
+                             f[e + 1]);
+              }
               w[8 * q2 + j] = pack_e4m3x4(f[0], f[1], f[2], f[3]);
             }
           }
@@ -707,13 +727,19 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
         }
       } else if (BN == 256 && !PAIR && p.epi == EPI_PIXEL) {
         // head layer 2 with the pixel shuffle (Sec. 3.4 Step 3): each 32-column chunk of the
-        // token's row is 32 / rs pixel rows of rs pixels, written as groups of 4 pixels
+        // token's row is 32 / rs pixel rows of rs pixels (rs a power of two), or at rs = 4 two
+        // channels. uint8 pixels leave in the widest store that a pixel row allows: neighbouring
+        // tokens' rows then fill whole sectors (14400 x 768 x 1024: 23.4 -> 21.5 us against groups
+        // of 4 pixels; fp32 31.3 -> 31.0, the shifts in place of divisions).
         const PixelEpi& px = p.pix;
         if (tile == 0 && warp == 2 && lane == 0 && px.step != nullptr) *px.step += 1;
         const int tau = row / px.tokens, l = row - tau * px.tokens;
         const bool out_row = row_ok && tau < px.frames;
         const int gy = l / px.gw, gx = l - gy * px.gw;
         const int rs = px.rs, rs2 = rs * rs, Wo = px.gw * rs, Ho = px.gh * rs;
+        const int lg = __ffs(rs) - 1;  // rs is 4, 8, 16 or 32
+        const size_t ch_px = static_cast<size_t>(px.frames) * Ho * Wo;
+        const size_t px0 = (static_cast<size_t>(tau) * Ho + gy * rs) * Wo + gx * rs;
 #pragma unroll 1
         for (int c = 32 * half; c < BN; c += 32 * kHalves) {
           const int col = n0 + c;
@@ -725,27 +751,52 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
           float bb[32];
           load32(p.bias + col, bb);
           if (!out_row) continue;
-          const int ch = col / rs2, rem = col - ch * rs2;
+          auto at = [&](int j) {  // place of column col + j (groups of at most rs columns)
+            const int cc = col + j, rem = cc & (rs2 - 1);
+            return px0 + static_cast<size_t>(cc >> (2 * lg)) * ch_px +
+                   static_cast<size_t>(rem >> lg) * Wo + (rem & (rs - 1));
+          };
+          if (px.u8) {
+            uint8_t* const out = static_cast<uint8_t*>(px.out);
+            uint32_t w[8];
 #pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            const int y = gy * rs + (rem + j) / rs, x = gx * rs + (rem + j) % rs;
-            const size_t o = ((static_cast<size_t>(ch) * px.frames + tau) * Ho + y) * Wo + x;
-            const float v0 = __uint_as_float(r[j]) + bb[j];
-            const float v1 = __uint_as_float(r[j + 1]) + bb[j + 1];
-            const float v2 = __uint_as_float(r[j + 2]) + bb[j + 2];
-            const float v3 = __uint_as_float(r[j + 3]) + bb[j + 3];
-            if (px.u8) {
-              *reinterpret_cast<uint32_t*>(static_cast<uint8_t*>(px.out) + o) =
-                  quant_u8(v0) | (quant_u8(v1) << 8) | (quant_u8(v2) << 16) |
-                  (quant_u8(v3) << 24);
+            for (int j = 0; j < 8; ++j) {
+              w[j] = 0;
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                w[j] |= quant_u8(__uint_as_float(r[4 * j + e]) + bb[4 * j + e]) << (8 * e);
+            }
+            if (rs >= 16) {
+              *reinterpret_cast<uint4*>(out + at(0)) = make_uint4(w[0], w[1], w[2], w[3]);
+              *reinterpret_cast<uint4*>(out + at(16)) = make_uint4(w[4], w[5], w[6], w[7]);
+            } else if (rs == 8) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                *reinterpret_cast<uint2*>(out + at(8 * j)) = make_uint2(w[2 * j], w[2 * j + 1]);
             } else {
-              *reinterpret_cast<float4*>(static_cast<float*>(px.out) + o) =
-                  make_float4(fminf(fmaxf(v0, -1.f), 1.f), fminf(fmaxf(v1, -1.f), 1.f),
-                              fminf(fmaxf(v2, -1.f), 1.f), fminf(fmaxf(v3, -1.f), 1.f));
+#pragma unroll
+              for (int j = 0; j < 8; ++j) *reinterpret_cast<uint32_t*>(out + at(4 * j)) = w[j];
+            }
+          } else {
+            float* const out = static_cast<float*>(px.out);
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+              float v[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                v[e] = fminf(fmaxf(__uint_as_float(r[j + e]) + bb[j + e], -1.f), 1.f);
+              *reinterpret_cast<float4*>(out + at(j)) = make_float4(v[0], v[1], v[2], v[3]);
             }
           }
         }
       } else {  // EPI_F32, EPI_RESID, EPI_TUP: fp32 slabs of 32 columns
+        // In the CTA's last tile every load has landed and every MMA has read its stage, so each
+        // slab gets a buffer of its own there and none waits for the store before it (1560 x 1024
+        // products of K = 1024 / 4096: 6.58 -> 6.38 and 13.97 -> 13.68 us; the two slabs of a GELU
+        // tile measured slower that way, 13.7 -> 14.1).
+        constexpr int kLastBufs = (BN / 32 + kHalves - 1) / kHalves;
+        static_assert(C::kEpiWarps * kLastBufs * 4096 <= C::kStgOffset, "last tile's buffers");
+        const bool last = tile + ctas >= tiles;
 #pragma unroll 1
         for (int c = 32 * half; c < BN; c += 32 * kHalves) {
           const int col = n0 + c;
@@ -767,7 +818,8 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
 #pragma unroll
             for (int j = 0; j < 32; ++j) w[j] = __float_as_uint(__uint_as_float(r[j]) + bb[j]);
           }
-          uint8_t* buf = acquire();
+          uint8_t* buf = last ? smem + ((warp - 2) * kLastBufs + (c / 32 - half) / kHalves) * 4096
+                              : acquire();
           put_row_sw128(buf, lane, w);
           publish();
           if (row0 < p.M && elect_one()) {

@@ -127,6 +127,15 @@ def test_linear_pixel_equals_linear_then_pixel_head(frames_in, frames, gh, gw, C
     assert torch.equal(got, want)
 
 
+@pytest.mark.parametrize("frames_in,frames,gh,gw,C,rs,u8", [
+    (2, 2, 9, 11, 4, 4, True), (2, 1, 9, 11, 4, 4, False),  # two channels per 32 columns
+    (2, 2, 9, 11, 3, 8, False), (3, 2, 9, 11, 3, 16, True), (1, 1, 7, 5, 3, 32, True),
+])
+def test_linear_pixel_stores_of_each_width(frames_in, frames, gh, gw, C, rs, u8):
+    """The pixel epilogue at every pixel-row length it takes: stores of 4, 8 or 16 codes."""
+    test_linear_pixel_equals_linear_then_pixel_head(frames_in, frames, gh, gw, C, rs, u8)
+
+
 def test_gelu_epilogue_is_the_exact_erf_gelu_at_bf16():
     """The GELU epilogue evaluates erf with Abramowitz & Stegun 7.1.26 (error <= 1.5e-7): on a
     grid of pre-activations from -8 to 8 (A holds x in one column, W picks it, the bias shifts
