@@ -327,16 +327,24 @@ __device__ __forceinline__ void head_rms(float (&v)[kDh], const float* g, float 
 // One thread does one (row, slot): its 64 values in order, as the sums over a head are. A block
 // stages kQkvBatch rows x up to kQkvSlots slots through shared memory (65 floats per unit: no bank
 // conflicts), so that global memory is read and written in whole lines: a thread reading its own
-// 256 bytes took 136 us forward and 89 us backward on average at 480p (36 and 52 staged). kQkvRows rows
-// per block.
-constexpr int kQkvBatch = 4, kQkvSlots = 32, kQkvRows = 16, kQkvPad = 65;
+// 256 bytes took 136 us forward and 89 us backward on average at 480p, staged 42 and 52. What is left
+// is a block's chain of load, sums and store, so the loads of a batch are issued together (36 / 34
+// us), the four rows of a slot sit in neighbouring threads (a warp then does one kind of slot: 31 /
+// 33) and a block takes one batch (kQkvRows rows): 22 / 28, for 1.1 us more in each sum of the
+// backward's partial rows; 8 rows a block 32 / 33.
+constexpr int kQkvBatch = 4, kQkvSlots = 32, kQkvRows = 4, kQkvPad = 65;
 constexpr int kQkvUnits = kQkvBatch * kQkvSlots;  // threads
+constexpr int kQkvLoads = kQkvSlots * kDh / (4 * kQkvUnits);  // 16-byte loads a thread and row
+__device__ __forceinline__ void put4(float* p, float4 v) {
+  p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w;
+}
 
 // QKV forward: q2 = RoPE(q0) (RMS with g2 first when qk_norm), k2 = RoPE(RMS(k0; gk)),
 // v1 = RMS(v0; g2) (v0 when qk_norm), in bf16. With qr non-null, also: q rows bf16 [M][N 64] (the
 // attention kernel's layout), and the real tokens' K bf16 [G][pitch][64] and V^T fp16
 // [G][64][pitch] without the padding rows (chunk c's Lu = Pc / Lp * L keys at c Lu ...), the keys
-// of the fused band attention. V^T leaves as the block's kQkvRows keys of each dimension.
+// of the fused band attention. V^T leaves as the block's kQkvRows
+// keys of each dimension.
 __global__ void __launch_bounds__(kQkvUnits)
     qkv_fwd_kernel(const float* __restrict__ qkv, QkvShape p, const float* __restrict__ gk,
                    const float* __restrict__ g2, float eps, Rope rp, bf16* __restrict__ q2,
@@ -348,19 +356,26 @@ __global__ void __launch_bounds__(kQkvUnits)
   const int slots = p.N + 2 * p.G, s0 = blockIdx.y * kQkvSlots;
   const int sc = min(kQkvSlots, slots - s0), units = kQkvBatch * sc;
   const int v0 = max(p.N + p.G, s0);  // first V slot of the block
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lu = tid / 16, lj = tid % 16 * 4;
+#pragma unroll 1
   for (int b = 0; b < kQkvRows / kQkvBatch; ++b) {
     const int row0 = blockIdx.x * kQkvRows + b * kQkvBatch;
-    for (int i = tid; i < units * 16; i += kQkvUnits) {
-      const int u = i / 16, j = i % 16 * 4;
-      const float4 x = *reinterpret_cast<const float4*>(
-          qkv + (static_cast<size_t>(row0 + u / sc) * slots + s0 + u % sc) * kDh + j);
-      float* px = xs + u * kQkvPad + j;
-      px[0] = x.x; px[1] = x.y; px[2] = x.z; px[3] = x.w;
-    }
+    float4 x[kQkvBatch][kQkvLoads];
+#pragma unroll
+    for (int i = 0; i < kQkvBatch; ++i)
+#pragma unroll
+      for (int k = 0; k < kQkvLoads; ++k)
+        if (lu + 8 * k < sc)
+          x[i][k] = *reinterpret_cast<const float4*>(
+              qkv + (static_cast<size_t>(row0 + i) * slots + s0 + lu + 8 * k) * kDh + lj);
+#pragma unroll
+    for (int i = 0; i < kQkvBatch; ++i)
+#pragma unroll
+      for (int k = 0; k < kQkvLoads; ++k)
+        if (lu + 8 * k < sc) put4(xs + ((lu + 8 * k) * kQkvBatch + i) * kQkvPad + lj, x[i][k]);
     __syncthreads();
     if (tid < units) {
-      const int row = row0 + tid / sc, slot = s0 + tid % sc;
+      const int row = row0 + tid % kQkvBatch, slot = s0 + tid / kQkvBatch;
       const int f = row / p.Lp, l = min(row % p.Lp, p.L - 1);  // padding rows: a real token's angles
       const int gy = l / p.gw, gx = l % p.gw;
       const bool is_q = slot < p.N, is_k = !is_q && slot < p.N + p.G;
@@ -383,9 +398,13 @@ __global__ void __launch_bounds__(kQkvUnits)
       for (int j = 0; j < kDh; ++j) px[j] = v[j];
     }
     __syncthreads();
-    for (int i = tid; i < units * 8; i += kQkvUnits) {  // eight values (16 bytes) each
-      const int u = i / 8, j = i % 8 * 8, row = row0 + u / sc, slot = s0 + u % sc;
-      const float* px = xs + u * kQkvPad + j;
+    // eight values (16 bytes) each
+#pragma unroll
+    for (int i = 0; i < kQkvBatch * kQkvLoads / 2; ++i) {
+      const int ri = i % kQkvBatch, su = tid / 8 + 16 * (i / kQkvBatch);
+      if (su >= sc) break;
+      const int j = tid % 8 * 8, row = row0 + ri, slot = s0 + su;
+      const float* px = xs + (su * kQkvBatch + ri) * kQkvPad + j;
       const uint2 lo = pack4(px[0], px[1], px[2], px[3]), hi = pack4(px[4], px[5], px[6], px[7]);
       const uint4 w = make_uint4(lo.x, lo.y, hi.x, hi.y);
       const bool is_q = slot < p.N, is_k = !is_q && slot < p.N + p.G;
@@ -407,11 +426,12 @@ __global__ void __launch_bounds__(kQkvUnits)
   }
   if (qr == nullptr) return;
   const int r0 = blockIdx.x * kQkvRows, nv = s0 + sc - v0;  // V slots of the block
-  for (int i = tid; i < nv * kDh * kQkvRows; i += kQkvUnits) {
-    const int r = r0 + i % kQkvRows, d = i / kQkvRows;  // d: dimension of group v0 - N - G + d / 64
-    if (r % p.Lp < p.L)
-      vtu[(static_cast<size_t>(v0 - p.N - p.G) * kDh + d) * pitch + p.key(r)] = vts[i];
-  }
+  const int r = r0 + tid % kQkvRows;
+  if (nv <= 0 || r % p.Lp >= p.L) return;
+  __half* const dst = vtu + static_cast<size_t>(v0 - p.N - p.G) * kDh * pitch + p.key(r);
+#pragma unroll 8
+  for (int d = tid / kQkvRows; d < nv * kDh; d += kQkvUnits / kQkvRows)  // of group d / 64
+    dst[static_cast<size_t>(d) * pitch] = vts[d * kQkvRows + tid % kQkvRows];
 }
 
 // RMS over one head, backward: x the pre-norm values in shared memory, overwritten by the gain's
@@ -449,29 +469,43 @@ __global__ void __launch_bounds__(kQkvUnits)
   float* const ds = sm + kQkvUnits * kQkvPad;
   const int slots = p.N + 2 * p.G, s0 = blockIdx.y * kQkvSlots;
   const int sc = min(kQkvSlots, slots - s0), units = kQkvBatch * sc, cols = sc * kDh;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lu = tid / 16, lj = tid % 16 * 4;
   auto normed = [&](int slot) {
     const bool is_q = slot < p.N, is_k = !is_q && slot < p.N + p.G;
     return is_k || (is_q ? p.qk_norm != 0 : p.qk_norm == 0);
   };
   // column pairs 2 tid, 2 tid + 1 (+ 256 k) of the block's slots
   float sb[16] = {}, st[16] = {};
+#pragma unroll 1
   for (int b = 0; b < kQkvRows / kQkvBatch; ++b) {
     const int row0 = blockIdx.x * kQkvRows + b * kQkvBatch;
-    for (int i = tid; i < units * 16; i += kQkvUnits) {
-      const int u = i / 16, j = i % 16 * 4, row = row0 + u / sc, slot = s0 + u % sc;
-      const float4 x = *reinterpret_cast<const float4*>(
-          qkv + (static_cast<size_t>(row) * slots + slot) * kDh + j);
-      const float* src = slot < p.N ? dq2 : (slot < p.N + p.G ? dk2 : dv1);
-      const float4 d = *reinterpret_cast<const float4*>(src + p.head_row(row, slot) * kDh + j);
-      float* px = xs + u * kQkvPad + j;
-      float* pd = ds + u * kQkvPad + j;
-      px[0] = x.x; px[1] = x.y; px[2] = x.z; px[3] = x.w;
-      pd[0] = d.x; pd[1] = d.y; pd[2] = d.z; pd[3] = d.w;
+#pragma unroll
+    for (int h = 0; h < kQkvBatch; h += 2) {
+      float4 x[2][kQkvLoads], d[2][kQkvLoads];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int k = 0; k < kQkvLoads; ++k) {
+          const int row = row0 + h + i, slot = s0 + lu + 8 * k;
+          if (lu + 8 * k >= sc) continue;
+          const float* src = slot < p.N ? dq2 : (slot < p.N + p.G ? dk2 : dv1);
+          x[i][k] = *reinterpret_cast<const float4*>(
+              qkv + (static_cast<size_t>(row) * slots + slot) * kDh + lj);
+          d[i][k] = *reinterpret_cast<const float4*>(src + p.head_row(row, slot) * kDh + lj);
+        }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int k = 0; k < kQkvLoads; ++k) {
+          if (lu + 8 * k >= sc) continue;
+          const int e = ((lu + 8 * k) * kQkvBatch + h + i) * kQkvPad + lj;
+          put4(xs + e, x[i][k]);
+          put4(ds + e, d[i][k]);
+        }
     }
     __syncthreads();
     if (tid < units) {
-      const int row = row0 + tid / sc, slot = s0 + tid % sc;
+      const int row = row0 + tid % kQkvBatch, slot = s0 + tid / kQkvBatch;
       const int f = row / p.Lp, l = min(row % p.Lp, p.L - 1);  // padding rows: a real token's angles
       const int gy = l / p.gw, gx = l % p.gw;
       const bool is_q = slot < p.N, is_k = !is_q && slot < p.N + p.G;
@@ -501,7 +535,7 @@ __global__ void __launch_bounds__(kQkvUnits)
       const bool t = normed(s0 + su);
 #pragma unroll
       for (int i = 0; i < kQkvBatch; ++i) {
-        const int e = (i * sc + su) * kQkvPad + j;
+        const int e = (su * kQkvBatch + i) * kQkvPad + j;
         const float a = ds[e], d = ds[e + 1];
         const __nv_bfloat162 v = __floats2bfloat162_rn(a, d);
         *reinterpret_cast<__nv_bfloat162*>(
@@ -538,6 +572,7 @@ __global__ void __launch_bounds__(kQkvUnits)
 }
 static_assert(kQkvUnits == 2 * kDh && kQkvRows % kQkvBatch == 0 &&
                   kQkvSlots * kDh <= 16 * kQkvUnits, "column phase");
+static_assert(kQkvUnits % kQkvRows == 0 && kQkvUnits == kQkvBatch * kQkvSlots, "V^T store");
 
 // ---------------------------------------------------------------- L1 term, pixel shuffle
 // L1 term of the pixels (reading T3: the mean of |x_hat - x| over the clip, unclamped output,
