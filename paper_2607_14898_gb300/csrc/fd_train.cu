@@ -1044,9 +1044,9 @@ fd_status fd_op_l1_pixel_bwd(const float* F, const float* target, int frames, in
   // one chunk of `frames` refined frames, rows unpadded (Lp = L)
   const fd::train::PixelGrid pg{1, frames, frames, L, L, grid_h, grid_w, channels, rs, inv_total};
   const int cols = channels * rs * rs;
-  const bool vec = rs % 4 == 0 && ((reinterpret_cast<uintptr_t>(F) |
-                                    reinterpret_cast<uintptr_t>(target) |
-                                    reinterpret_cast<uintptr_t>(dF)) & 15u) == 0;
+  const bool vec = rs % 4 == 0 && L <= 65535 * fd::train::kRowBlock / frames &&  // grid y
+                   ((reinterpret_cast<uintptr_t>(F) | reinterpret_cast<uintptr_t>(target) |
+                     reinterpret_cast<uintptr_t>(dF)) & 15u) == 0;
   int parts = blocks;
   if (vec) {  // no more partial sums than the caller's scratch holds: a row has cols >= 16 elements
     const int strips = (cols + 1023) / 1024;

@@ -275,3 +275,69 @@ def test_attention_backward_tiles(lat_h, lat_w, chunks, window, r_t, heads, grou
         # the tensor's own scale plus fp32 noise of the whole step
         err, scale = float((g - ref).norm()), float(ref.norm())
         assert err <= GRAD_REL * scale + 1e-6, (k, err, scale)
+
+
+def test_qkv_slots_past_one_block():
+    """Heads and KV groups of more slots (12 + 2 x 12) than one block of the QKV kernels takes."""
+    test_attention_backward_tiles(6, 10, 2, 2, 1, 12, 12, True)
+
+
+@pytest.mark.parametrize("M,D,off", [
+    (1, 64, 0), (17, 64, 0),           # fewer rows than the thread groups of a narrow D
+    (5, 33, 0), (16, 1025, 0),         # D no multiple of 4
+    (33, 100, 0), (33, 100, 1),        # a multiple; the same off 16 bytes
+])
+def test_rmsnorm_backward_widths_and_alignments(M, D, off):
+    """fd_op_rmsnorm_bwd's vector and scalar columns (bound as in test_rmsnorm_backward_kernel)."""
+    from oracle.backward import rms_norm_bwd
+    from helpers import randn
+
+    def place(a):  # `off` floats into a buffer
+        t = torch.empty(a.size + off, device="cuda")[off:].view(a.shape)
+        t.copy_(torch.from_numpy(a))
+        return t
+    x, g, dy = randn((M, D), M + D, 2.0), 1 + randn((D,), M + D + 1, 0.02), randn((M, D), M + D + 2)
+    dx, dg = place(np.zeros((M, D), np.float32)), torch.empty(D, device="cuda")
+    fdp.op_rmsnorm_bwd(place(x), torch.from_numpy(g).cuda(), place(dy), 1e-6, dx, dg)
+    torch.cuda.synchronize()
+    want = rms_norm_bwd(torch.from_numpy(x).double(), torch.from_numpy(g).double(), 1e-6,
+                        torch.from_numpy(dy).double())
+    for got, ref in zip((dx, dg), want):
+        assert float((got.cpu().double() - ref).abs().max()) < 2e-5 * float(ref.abs().max())
+
+
+@pytest.mark.parametrize("n,off", [(3, 0), (4096, 0), (4096, 1), (4098, 0)])
+def test_gelu_backward_lengths_and_alignments(n, off):
+    """fd_op_gelu_bwd's vector and scalar forms give the oracle's values (bounds as in
+    test_gelu_backward_kernel)."""
+    from oracle.backward import gelu_bwd
+    z = torch.linspace(-9, 9, n, dtype=torch.float32)
+    da = torch.cos(torch.arange(n, dtype=torch.float32))
+    zd, dad, dz = (torch.zeros(n + off, device="cuda")[off:] for _ in range(3))
+    dz16 = torch.zeros(n, dtype=torch.bfloat16, device="cuda")
+    zd.copy_(z)
+    dad.copy_(da)
+    fdp.op_gelu_bwd(zd, dad, dz, dz16)
+    torch.cuda.synchronize()
+    assert float((dz.cpu().double() - gelu_bwd(z.double(), da.double())).abs().max()) < 2e-6
+    assert torch.equal(dz16.cpu(), dz.cpu().to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("frames,gh,gw,C,rs", [(2, 3, 5, 3, 6), (1, 1, 1, 1, 4), (3, 5, 7, 3, 20)])
+def test_l1_pixel_backward_pixel_rows(frames, gh, gw, C, rs):
+    """fd_op_l1_pixel_bwd with pixel rows that are no multiple of 4 (element by element), with a
+    single token, and with more than 1024 columns (two strips). Loss bound: fp32 terms summed in a
+    tree and in fp64."""
+    from oracle.backward import l1_bwd, pixel_shuffle_bwd
+    from helpers import randn
+    F = randn((frames * gh * gw, C * rs * rs), 5, 0.3)
+    x = randn((C, frames, gh * rs, gw * rs), 6, 0.3)
+    dF, loss = torch.empty(F.shape, device="cuda"), torch.zeros(1, device="cuda")
+    fdp.op_l1_pixel_bwd(torch.from_numpy(F).cuda(), torch.from_numpy(x).cuda(), frames, gh, gw,
+                        C, rs, dF, loss)
+    torch.cuda.synchronize()
+    pix = oracle.pixel_shuffle(torch.from_numpy(F).double(), frames, gh, gw, C, rs)
+    want = float((pix - torch.from_numpy(x).double()).abs().mean())
+    assert abs(float(loss.item()) - want) <= 1e-6 * want
+    want_dF = pixel_shuffle_bwd(l1_bwd(pix, x, pix.numel()), frames, gh, gw, C, rs)
+    assert float((dF.cpu().double() - want_dF).abs().max()) <= 1e-7 / pix.numel()
