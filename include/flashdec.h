@@ -341,10 +341,11 @@ enum fd_train_kind {
   FD_TK_LINEAR = 0,     /* forward products of the linears (embedding, blocks, upsampling, head) */
   FD_TK_DGRAD = 1,      /* their input gradients, dX = dY W */
   FD_TK_WGRAD = 2,      /* their weight gradients, dW = dY^T X */
-  FD_TK_ATTN_GEMM = 3,  /* the attention's products: S = Q K^T (forward and recomputed), P V,
-                           dP = dO V^T, dQ = dS K, dK = dS^T Q, dV = P^T dO */
-  FD_TK_SOFTMAX = 4,    /* band softmax, row dot delta = rowsum(dO o O), softmax backward */
-  FD_TK_TRANSPOSE = 5,  /* operand transposes for the products */
+  FD_TK_ATTN_GEMM = 3,  /* the attention, forward and backward: S = Q K^T (also recomputed), P V,
+                           dP = dO V^T, dQ = dS K, dK = dS^T Q, dV = P^T dO, with the softmax and
+                           its backward where they are fused */
+  FD_TK_SOFTMAX = 4,    /* band softmax of a materialised forward, delta = rowsum(dO o O) */
+  FD_TK_TRANSPOSE = 5,  /* operand transposes for the products (a materialised forward's) */
   FD_TK_NORM = 6,       /* RMSNorm forward / backward, KV-norm (QK-norm) + 3D-RoPE fwd / bwd */
   FD_TK_POINTWISE = 7,  /* bf16 casts, GELU forward / backward, copies, column sums, the
                            PixelUnshuffle, upsampling permutes and the L1 loss */

@@ -289,9 +289,9 @@ __device__ __forceinline__ uint32_t pack_e4m3x4(float f0, float f1, float f2, fl
 }
 // ---- MMAs and commits issued by one lane of a converged warp: the whole warp runs the issue
 // loop and elect.sync picks the lane (always the same one, so its commits track its own
-// MMAs). On the GB300 a lone lane inside a divergent branch issued tcgen05.mma one per
-// 137-158 cycles, an elected lane of a converged warp one per 125-126 (M = 128, N = 64 / 128);
-// the GEMM's issuer uses this form (the attention's issuers measured faster as lone lanes).
+// MMAs). With a warp index that the compiler knows to be uniform (warp_index) the MMAs leave at the
+// tensor or shared-memory rate, 48 / 64 / 128 cycles at M = 128, N = 64 / 128 / 256; a lone lane
+// inside a divergent branch took 137-158 whatever N.
 __device__ __forceinline__ void mma_commit_w(uint32_t bar) {
   asm volatile(
       "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t"
@@ -317,7 +317,6 @@ __device__ __forceinline__ void mma_commit_pair_w(uint32_t bar, uint16_t cta_mas
 // issued by the even CTA: M = 256 (A rows 0..127 from this CTA's shared memory, 128..255 from
 // the peer's at the same offset), B's N rows split in halves the same way; each CTA's TMEM
 // receives its 128 rows of D.
-// Measured on the GB300 at 104-124 cycles per MMA against 125-126 for separate elected MMAs.
 #define FD_MMA4_BODY(KIND, GROUP, O1, O2, O3)                                              \
   "{\n\t.reg .pred p, q, e;\n\t.reg .b32 r;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"     \
   "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, %4, %4;\n\t"                                   \
@@ -370,8 +369,8 @@ __device__ __forceinline__ void mma4_bf16_mn_pair_w(uint32_t d_tmem, uint64_t ad
                : "memory");
 }
 #undef FD_MMA4_BODY
-// The same four-MMA block issued by the calling thread alone (the attention's issuers: a lone
-// lane; measured 142 against 158 cycles per MMA for four separate asm statements).
+// The same four-MMA block issued by the calling thread alone (the attention's issuers call it under
+// one elect_one for the MMAs and their commits).
 __device__ __forceinline__ void mma4_bf16_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                              uint32_t idesc, uint32_t accumulate) {
   asm volatile(

@@ -337,8 +337,9 @@ struct Linear {
 };
 
 // Launch shape of an M x N x K product. CTA pairs (256 x 256 tiles, each SM holding half of W)
-// measured 4-10 % faster than the best single-CTA tile once there are at least 2.5 rounds of
-// pair tiles, and slower on the smaller products, where a tile's fixed costs dominate; there
+// measured 3-16 % faster than the best single-CTA tile once there are at least 2.5 rounds of
+// pair tiles (6240 x 4096 x 1024 with GELU 39.4 -> 33.2 us, 13312 x 1024 x 4096 73.5 -> 64.3), and
+// slower on the smaller products, where a tile's fixed costs dominate; there
 // the single-CTA width model of pick_bn_step (which matches the measured best width) decides.
 struct TileChoice {
   int bn;
