@@ -455,6 +455,7 @@ __global__ void __launch_bounds__(attn::kThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (elect_one()) mbar_arrive(bar(kBarSFree + x));  // S_X may receive the next scores
+      __syncwarp();  // the turns below are taken by converged warps
       const int valid = n_keys - cur.kb * 128;
       if (valid < 128) {  // ragged last key block (warp-uniform branch)
 #pragma unroll

@@ -296,6 +296,7 @@ __global__ void __launch_bounds__(attn_bwd::kThreads, 1)
       }
       if (j > 0 && !mbar_wait_warp(bar(kPFree), (j - 1) & 1, p.err, ERR_WAIT_MMA)) break;
       tc_fence_after();
+      __syncwarp();  // block 0 waits for nothing after the elected arrive above
       tmem_st_32x32b_x16(lanes + kColDs + 16u * hc, pd);
       if constexpr (KV) tmem_st_32x32b_x16(lanes + kColP + 16u * hc, pp);
       tmem_st_wait();

@@ -179,8 +179,12 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// every thread of every CTA of the cluster arrives, then waits (release / acquire)
+// every thread of every CTA of the cluster arrives, then waits (release / acquire). Like the TMEM
+// allocations, it starts by reconverging its warp: all lanes have to execute such an .aligned
+// instruction together, and the code before it may have branched on one lane (the one that
+// initialises the barriers).
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
                ::: "memory");
 }
@@ -208,6 +212,7 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
 }
 // the pair allocates (and frees) the same TMEM columns in both SMs: one warp of each CTA
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem),
                "r"(ncols)
                : "memory");
@@ -263,6 +268,7 @@ __device__ __forceinline__ void bulk_wait_read_0() {
 
 // ---------------------------------------------------------------- tcgen05
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem),
                "r"(ncols)
                : "memory");
@@ -482,7 +488,9 @@ __device__ __forceinline__ void tmem_st_32x32b_x8(uint32_t taddr, const uint32_t
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
       : "memory");
 }
-// named barrier among `count` threads (ids 1..15; id 0 is __syncthreads)
+// named barrier among `count` threads (ids 1..15; id 0 is __syncthreads), taken by converged warps:
+// the caller reconverges after a branch on one lane. A __syncwarp here held back the arithmetic
+// around the attention's turns (53 -> 60 us at 1560 x 6240, 2860 -> 3300 at 14400 x 57600).
 __device__ __forceinline__ void named_barrier(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
