@@ -253,6 +253,11 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
     }
   }
   grid_dep_wait();  // inputs written by the previous kernel; TMEM freed by its CTAs
+  // A decode's last launch advances the chunk counter (which no thread of it reads), also in a
+  // chunk that a wait below stops: the host's count has advanced as well.
+  if (BN == 256 && !PAIR && QKV == 0 && !DS && !MN && p.epi == EPI_PIXEL && blockIdx.x == 0 &&
+      threadIdx.x == blockDim.x - 1 && p.pix.step != nullptr)
+    *p.pix.step += 1;
   // The producer needs no TMEM: it goes on to its loads while the others wait for the allocation
   // (and for the barriers, which it has initialised).
   constexpr int kReady = 1;
@@ -732,7 +737,6 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(QKV), 1)
         // tokens' rows then fill whole sectors (14400 x 768 x 1024: 23.4 -> 21.5 us against groups
         // of 4 pixels; fp32 31.3 -> 31.0, the shifts in place of divisions).
         const PixelEpi& px = p.pix;
-        if (tile == 0 && warp == 2 && lane == 0 && px.step != nullptr) *px.step += 1;
         const int tau = row / px.tokens, l = row - tau * px.tokens;
         const bool out_row = row_ok && tau < px.frames;
         const int gy = l / px.gw, gx = l - gy * px.gw;

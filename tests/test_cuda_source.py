@@ -1,6 +1,7 @@
-"""Checks of the CUDA sources that no run can make. An .aligned instruction (the barriers, TMEM
+"""Checks of the CUDA sources that no run can make: of paths that only a stopped wait takes, and of
+code that a compiler may happen to make right. An .aligned instruction (the barriers, TMEM
 allocations and TMEM stores among them) has to be reached by all lanes of a warp together: code that
-branches on one lane before it reconverges first, and does not rely on the compiler to."""
+branches on one lane before it reconverges first."""
 import os
 import re
 
@@ -44,3 +45,11 @@ def test_attention_backward_stores_to_tmem_from_converged_warps():
     part = between(source("fd_attn_bwd.cu"), "mbar_arrive(bar(kSFree))",
                    "tmem_st_32x32b_x16(lanes + kColDs")
     assert "\n      __syncwarp();" in part
+
+
+def test_chunk_counter_advances_before_any_wait_of_the_last_launch():
+    """The decode's last launch advances the device's chunk counter whether or not its waits (for
+    loads, MMAs, the accumulator) come to their end, as the host advances its own."""
+    src = source("fd_gemm_kernel.cuh")
+    body = src[src.index("gemm_kernel(const __grid_constant__"):]
+    assert body.index("grid_dep_wait();") < body.index("pix.step += 1") < body.index("mbar_wait")
