@@ -208,3 +208,14 @@ def test_library_is_rebuilt_when_a_source_or_header_changes():
     finally:
         os.utime(hdr, (st.st_atime, st.st_mtime))
     assert b.up_to_date()
+
+
+def test_current_stream_without_the_private_function(monkeypatch):
+    """A torch that does not have the private function the binding reads the current stream with:
+    the public call gives the same pointer."""
+    import types
+    torch = pytest.importorskip("torch")
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    assert fdp._stream_ptr(None) == 77
