@@ -185,6 +185,21 @@ fd_status fd_op_scores_bwd(int M, int N, const void* Q, const void* dO, const vo
                            const void* V, const float* lse, const float* delta, int Pc, int Lp,
                            int L, void* dS, void* dST, void* PT, int* err_dev, void* stream);
 
+/* The training step's attention backward over a clip of T query chunks (fd_train_step's two
+ * launches, Sec. 3.3): query chunk i sees key chunks max(0, i - W + 1) .. i, heads n the KV group
+ * n / (N / G). q, dO bf16 [T][N][Pc][64]; k, v bf16 [G][T Pc][64]; lse, delta fp32 [T][N][Pc]: each
+ * row's log-sum-exp of its scores q k / sqrt(64) and rowsum(dO o O). Pc rows per chunk are whole
+ * frames of Lp rows, of which the first L are tokens: keys past them take no part, and a padding
+ * query row has lse = +inf and dO = 0. With P = exp(S / sqrt(64) - lse), dP = dO V^T and
+ * dS = P (dP - delta) / sqrt(64): dq = dS K (fp32 [T][N][Pc][64]), dk = dS^T Q and dv = P^T dO
+ * (fp32 [G][T Pc][64], summed over the group's heads and the query chunks, hs heads of a chunk to an
+ * accumulator chain). Lp % 128 == 0, Pc % Lp == 0, (N / G) % hs == 0; 16-byte aligned.
+ * Errors: FD_ERR_INVALID_ARG, FD_ERR_CUDA; err_dev as for fd_op_linear. */
+fd_status fd_op_attention_bwd(int T, int N, int G, int W, int Pc, int Lp, int L, int hs,
+                              const void* q, const void* dO, const void* k, const void* v,
+                              const float* lse, const float* delta, float* dq, float* dk, float* dv,
+                              int* err_dev, void* stream);
+
 /* RMSNorm backward (the derivative of y = x r g, r = (mean(x^2) + eps)^(-1/2), Sec. 3.2):
  * dx = r (dy g) - x r^3 sum_j(dy_j g_j x_j) / D and dg = sum over rows of dy x r.
  * x, dy, dx fp32 [M][D]; g, dg fp32 [D]; work: fp32 [M][D] scratch of the caller. */

@@ -319,7 +319,7 @@ cudaError_t gemm_wgrad(int n_out, int n_in, int rows, const __nv_bfloat16* dY,
 cudaError_t scores_bwd(int M, int N, const __nv_bfloat16* Q, const __nv_bfloat16* dO, int ldq,
                        const __nv_bfloat16* K, const __nv_bfloat16* V, int ldk, const DsEpi& ds,
                        int* err, cudaStream_t s);
-// the same launch with its maps made from the tensors' addresses
+// launch_attention_bwd with its maps made from the tensors' addresses (16-byte aligned)
 cudaError_t attention_bwd(const __nv_bfloat16* q, const __nv_bfloat16* dO, const __nv_bfloat16* k,
                           const __nv_bfloat16* v, const AttnBwdParams& p, float* dq, float* dk,
                           float* dv, cudaStream_t s);

@@ -989,6 +989,24 @@ fd_status fd_op_scores_bwd(int M, int N, const void* Q, const void* dO, const vo
   return e == cudaSuccess ? FD_OK : FD_ERR_CUDA;
 }
 
+fd_status fd_op_attention_bwd(int T, int N, int G, int W, int Pc, int Lp, int L, int hs,
+                              const void* q, const void* dO, const void* k, const void* v,
+                              const float* lse, const float* delta, float* dq, float* dk, float* dv,
+                              int* err_dev, void* stream) {
+  if (!err_dev || T < 1 || N < 1 || G < 1 || N % G || W < 1 || Lp < 128 || Lp % 128 || Pc < Lp ||
+      Pc % Lp || L < 1 || L > Lp || hs < 1 || N / G % hs)
+    return FD_ERR_INVALID_ARG;
+  if (static_cast<long long>(T) * Pc > (1LL << 30) / N) return FD_ERR_INVALID_ARG;  // int rows
+  const void* const ptrs[9] = {q, dO, k, v, lse, delta, dq, dk, dv};
+  for (const void* ptr : ptrs)
+    if (!ptr || reinterpret_cast<uintptr_t>(ptr) & 15u) return FD_ERR_INVALID_ARG;
+  const fd::AttnBwdParams p{lse, delta, nullptr, nullptr, T, N, G, W, Pc, Lp, L, T * Pc, hs, err_dev};
+  const cudaError_t e = fd::attention_bwd(
+      static_cast<const bf16*>(q), static_cast<const bf16*>(dO), static_cast<const bf16*>(k),
+      static_cast<const bf16*>(v), p, dq, dk, dv, static_cast<cudaStream_t>(stream));
+  return e == cudaSuccess ? FD_OK : FD_ERR_CUDA;
+}
+
 fd_status fd_op_rmsnorm_bwd(const float* x, const float* g, const float* dy, int M, int D,
                             float eps, float* dx, float* dg, float* work, void* stream) {
   if (!x || !g || !dy || !dx || !dg || !work || M < 1 || D < 1 || D > 65536)

@@ -84,6 +84,7 @@ _SIGS = {
     "fd_train_grad_elems": (ctypes.c_size_t, [ctypes.POINTER(fd_config)]),
     "fd_op_linear_pixel": (_I, [_I, _I, _P, _P, _P, _I, _I, _I, _I, _I, _I, _P, _P, _P]),
     "fd_op_rmsnorm_bwd": (_I, [_P, _P, _P, _I, _I, _F, _P, _P, _P, _P]),
+    "fd_op_attention_bwd": (_I, [_I] * 8 + [_P] * 11),
     "fd_op_scores_bwd": (_I, [_I, _I, _P, _P, _P, _P, _P, _P, _I, _I, _I, _P, _P, _P, _P, _P]),
     "fd_op_gelu_bwd": (_I, [_P, _P, ctypes.c_int64, _P, _P, _P]),
     "fd_op_l1_pixel_bwd": (_I, [_P, _P, _I, _I, _I, _I, _I, _P, _P, _P, _P]),
@@ -608,6 +609,16 @@ def op_scores_bwd(Q, dO, K, V, lse, delta, Pc, Lp, L, dS, dST, PT, err=None,
     _check(lib().fd_op_scores_bwd(M, N, _ptr(Q), _ptr(dO), _ptr(K), _ptr(V), _ptr(lse),
                                   _ptr(delta), Pc, Lp, L, _ptr(dS), _ptr(dST), _ptr(PT), _ptr(err),
                                   _stream_ptr(stream)), "fd_op_scores_bwd")
+
+
+def op_attention_bwd(q, dO, k, v, lse, delta, W, Lp, L, hs, dq, dk, dv, err=None,
+                     stream=None) -> None:
+    """The training step's attention backward (fd_op_attention_bwd): q, dO [T][N][Pc][64]; k, v
+    [G][T Pc][64]."""
+    T, N, Pc = q.shape[:3]
+    _check(lib().fd_op_attention_bwd(T, N, k.shape[0], W, Pc, Lp, L, hs, _ptr(q), _ptr(dO), _ptr(k),
+                                     _ptr(v), _ptr(lse), _ptr(delta), _ptr(dq), _ptr(dk), _ptr(dv),
+                                     _ptr(err), _stream_ptr(stream)), "fd_op_attention_bwd")
 
 
 def op_rmsnorm_bwd(x, g, dy, eps, dx, dg, stream=None) -> None:

@@ -219,3 +219,18 @@ def test_current_stream_without_the_private_function(monkeypatch):
     monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
     assert fdp._stream_ptr(None) == 77
+
+
+def test_attention_bwd_refuses_shapes_it_cannot_tile():
+    """fd_op_attention_bwd checks its shapes before it launches anything."""
+    L = fdp.lib()
+    buf = np.zeros(4096, np.uint8)
+    at = (buf.ctypes.data + 15) // 16 * 16
+    ok = dict(T=2, N=4, G=2, W=2, Pc=256, Lp=128, L=100, hs=2)
+    for bad in (dict(G=3), dict(Lp=96, Pc=96, L=90), dict(Pc=192), dict(L=129), dict(L=0), dict(hs=3),
+                dict(W=0), dict(T=1 << 22, Pc=1 << 14)):
+        c = {**ok, **bad}
+        ptrs = [ctypes.c_void_p(at)] * 10 + [None]
+        assert L.fd_op_attention_bwd(*(c[n] for n in ok), *ptrs) == 1, bad
+    ptrs = [ctypes.c_void_p(at + 4)] + [ctypes.c_void_p(at)] * 9 + [None]
+    assert L.fd_op_attention_bwd(*ok.values(), *ptrs) == 1  # q off 16 bytes

@@ -341,3 +341,88 @@ def test_l1_pixel_backward_pixel_rows(frames, gh, gw, C, rs):
     assert abs(float(loss.item()) - want) <= 1e-6 * want
     want_dF = pixel_shuffle_bwd(l1_bwd(pix, x, pix.numel()), frames, gh, gw, C, rs)
     assert float((dF.cpu().double() - want_dF).abs().max()) <= 1e-7 / pix.numel()
+
+
+@pytest.mark.parametrize("T,N,G,W,frames,L,hs", [
+    (2, 2, 2, 2, 1, 2, 1),      # two tokens per frame (126 padding rows), one head per group
+    (3, 4, 1, 2, 1, 128, 4),    # no padding; every head of a chunk in one accumulator chain
+    (3, 4, 2, 3, 2, 129, 2),    # one token in a frame's second tile; two frames per chunk
+    (3, 4, 2, 3, 2, 129, 1),    # the same, each head its own chain
+    (2, 2, 1, 4, 4, 255, 2),    # one padding row per frame; window longer than the clip
+    (5, 6, 1, 2, 1, 100, 3),    # two chains per chunk and group
+    (4, 8, 1, 4, 1, 200, 8),    # chains of more blocks than the load ring holds
+])
+def test_attention_backward_kernels(T, N, G, W, frames, L, hs):
+    """fd_op_attention_bwd, the step's dQ and dK / dV launches, against oracle.attention_bwd in fp64,
+    each tensor by itself. Bar: the kernels round P and dS to bf16 and do the rest in fp32, so
+    1.5 times the movement that these two roundings alone cause in fp64, plus 1e-4 (64-term fp32
+    sums, exponents below 8: a few 1e-6 per score). Padding rows get exact zeros."""
+    from helpers import bf16_values, randn
+    Lp = (L + 127) // 128 * 128
+    Pc, hpg = frames * Lp, N // G
+    M = T * Pc
+    pos = torch.arange(M)
+    live, chunk = pos % Lp < L, pos // Pc
+    allowed = live[None] & (chunk[None] <= chunk[:, None]) & (chunk[None] > chunk[:, None] - W)
+    t = lambda shape, i: torch.from_numpy(bf16_values(randn(shape, 1000 * T + 10 * L + i))).double()
+    q, k, v, do = t((N, M, 64), 0), t((G, M, 64), 1), t((G, M, 64), 2), t((N, M, 64), 3)
+    do[:, ~live] = 0.0
+    kk, vv = k.repeat_interleave(hpg, 0), v.repeat_interleave(hpg, 0)
+    s = (q @ kk.transpose(1, 2) / 8.0).masked_fill(~allowed, float("-inf"))
+    lse = torch.logsumexp(s, -1)
+    p = torch.softmax(s, -1)
+    delta = (do * (p @ vv)).sum(-1)
+    want = dict(zip(("dq", "dk", "dv"), oracle_bwd.attention_bwd(q, k, v, do, allowed)))
+    # the movement of the bf16 P and dS
+    bf = lambda x: x.to(torch.bfloat16).double()
+    ds = bf(p * (do @ vv.transpose(1, 2) - delta[..., None]) / 8.0)
+    group = lambda x: x.reshape(G, hpg, M, 64).sum(1)
+    moved = {"dq": ds @ kk, "dk": group(ds.transpose(1, 2) @ q),
+             "dv": group(bf(p).transpose(1, 2) @ do)}
+    rows = lambda x: x.reshape(N, T, Pc, *x.shape[2:]).transpose(0, 1).contiguous().cuda()
+    lse[:, ~live] = float("inf")
+    got = {"dq": torch.full((T, N, Pc, 64), float("nan"), device="cuda"),
+           "dk": torch.full((G, M, 64), float("nan"), device="cuda"),
+           "dv": torch.full((G, M, 64), float("nan"), device="cuda")}
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    fdp.op_attention_bwd(rows(q.bfloat16()), rows(do.bfloat16()), k.bfloat16().cuda(),
+                         v.bfloat16().cuda(), rows(lse.float()), rows(delta.float()), W, Lp, L, hs,
+                         got["dq"], got["dk"], got["dv"], err=err)
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    got["dq"] = got["dq"].transpose(0, 1).reshape(N, M, 64)
+    for name, x in got.items():
+        x, ref = x.cpu().double(), want[name]
+        assert float(x[:, ~live].abs().sum()) == 0.0, name
+        bar = 1.5 * float((moved[name] - ref).norm()) + 1e-4 * float(ref.norm())
+        assert float((x - ref).norm()) <= bar, (name, float((x - ref).norm()), bar)
+
+
+@pytest.mark.parametrize("lat_h,lat_w,chunks,window,r_t,heads,groups,qk", [
+    (16, 16, 1, 1, 1, 2, 1, False), (16, 32, 3, 2, 1, 4, 1, True), (6, 86, 3, 3, 2, 4, 2, False),
+    (30, 34, 2, 4, 4, 2, 2, False), (20, 26, 5, 3, 4, 4, 2, False),
+])
+def test_query_key_and_value_gradients_each_by_itself(lat_h, lat_w, chunks, window, r_t, heads,
+                                                      groups, qk):
+    """The step's gradients that dQ, dK and dV reach, each held to its own norm: the Q, K and V rows
+    of the QKV weight and bias (V's are several times larger than Q's and K's, and would hide them)
+    and the gains. Bars: with every matrix operand of the step rounded to bf16 / fp16 (forward, and
+    dY, dO, P, dS backward) the fp64 oracle moves these by at most 0.71 % on these clips, K's bias
+    rows by 2.1 % (sums of a key's dS over all queries nearly cancel); 3 times that."""
+    cfg = synth.FDConfig(latent_h=lat_h, latent_w=lat_w, patch=2, hidden=64 * heads, heads=heads,
+                         kv_groups=groups, n_blocks=1, n_refine=1 if r_t > 1 else 0,
+                         window=window, r_t=r_t, qk_norm=qk, chunks=chunks, name="qkv")
+    w, z = synth.make_weights(cfg), synth.make_latents(cfg)
+    x = synth.make_target_pixels(cfg, min_abs=0.3)
+    _, g_ref = training_step_explicit(cfg, w, z, x)
+    got = split(cfg, gpu_step(cfg, w, z, x)[1])
+    nq, nk = 64 * heads, 64 * groups
+    for name, ref in g_ref.items():
+        if "qkv." not in name and not name.endswith("norm.g"):
+            continue
+        parts = {"": slice(None)} if "qkv." not in name else {
+            "Q": slice(0, nq), "K": slice(nq, nq + nk), "V": slice(nq + nk, None)}
+        for part, rows in parts.items():
+            a, b = got[name][rows], ref.reshape(got[name].shape)[rows]
+            bar = 6.3e-2 if name.endswith("qkv.b") and part == "K" else 2.1e-2
+            assert float((a - b).norm()) <= bar * float(b.norm()), (name, part)
