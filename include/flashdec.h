@@ -259,7 +259,10 @@ fd_status fd_sync_status(fd_handle h);
 /* Static description of a status code. */
 const char* fd_status_str(fd_status s);
 
-/* Kernel kinds of the decode path, for the per-kernel profile. */
+/* Kernel kinds of the decode path, for the per-kernel profile. FD_K_UNSHUFFLE is a chunk's first
+ * launch, which also writes its RoPE tables, and the last one (FD_K_HEAD2 or FD_K_PIXEL) advances
+ * the chunk counter: FD_K_ROPE and FD_K_ADVANCE, once launches of their own, keep their values and
+ * count nothing. */
 typedef enum {
   FD_K_UNSHUFFLE = 0, FD_K_EMBED = 1, FD_K_RMSNORM = 2, FD_K_QKV = 3, FD_K_ATTN_B = 4,
   FD_K_ATTN_R = 5, FD_K_OUT = 6, FD_K_MLP1 = 7, FD_K_MLP2 = 8, FD_K_TUP = 9, FD_K_HEAD1 = 10,
@@ -274,7 +277,8 @@ typedef enum {
 fd_status fd_profile_enable(fd_handle h, int enable);
 fd_status fd_profile_collect(fd_handle h, int64_t* launches, double* ms);
 
-/* Number of kernels this handle has launched since fd_create. */
+/* Number of kernels this handle has launched since fd_create. fd_decode_batch launches each kernel
+ * for all its streams at once, and counts and profiles it on the call's first handle. */
 int64_t fd_launch_count(fd_handle h);
 
 /* Streaming state, for checkpoint / resume and for moving a stream to another handle (no
@@ -345,15 +349,18 @@ enum fd_train_kind {
                            dP = dO V^T, dQ = dS K, dK = dS^T Q, dV = P^T dO, with the softmax and
                            its backward where they are fused */
   FD_TK_SOFTMAX = 4,    /* band softmax of a materialised forward, delta = rowsum(dO o O) */
-  FD_TK_TRANSPOSE = 5,  /* operand transposes for the products (a materialised forward's) */
+  FD_TK_TRANSPOSE = 5,  /* operand transposes for the products (a materialised forward's, and the
+                           weight gradient's of an input that is no multiple of 64 wide) */
   FD_TK_NORM = 6,       /* RMSNorm forward / backward, KV-norm (QK-norm) + 3D-RoPE fwd / bwd */
-  FD_TK_POINTWISE = 7,  /* bf16 casts, GELU forward / backward, copies, column sums, the
-                           PixelUnshuffle, upsampling permutes and the L1 loss */
+  FD_TK_POINTWISE = 7,  /* GELU / gated SiLU forward and backward, the upsampling's backward and
+                           the L1 loss (with their bf16 copies and column sums), copies, the
+                           PixelUnshuffle */
   FD_TK_COUNT = 8
 };
 /* Per-kernel profile of the training step: while enabled, every launch of fd_train_step is
- * bracketed by CUDA events on its stream. fd_train_profile_collect synchronises the device,
- * adds each kind's launch count and device milliseconds into launches[FD_TK_COUNT] /
+ * bracketed by CUDA events on its stream (one bracket, counted once, for a kernel and the sum of its
+ * partial rows, and for the attention backward's two launches). fd_train_profile_collect
+ * synchronises the device, adds each kind's launch count and device milliseconds into launches[FD_TK_COUNT] /
  * ms[FD_TK_COUNT] (the caller zeroes them) and releases the recorded events.
  * Errors: FD_ERR_INVALID_ARG (null arguments), FD_ERR_CUDA. */
 fd_status fd_train_profile_enable(fd_trainer tr, int enable);

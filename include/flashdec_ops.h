@@ -192,8 +192,8 @@ fd_status fd_op_scores_bwd(int M, int N, const void* Q, const void* dO, const vo
  * frames of Lp rows, of which the first L are tokens: keys past them take no part, and a padding
  * query row has lse = +inf and dO = 0. With P = exp(S / sqrt(64) - lse), dP = dO V^T and
  * dS = P (dP - delta) / sqrt(64): dq = dS K (fp32 [T][N][Pc][64]), dk = dS^T Q and dv = P^T dO
- * (fp32 [G][T Pc][64], summed over the group's heads and the query chunks, hs heads of a chunk to an
- * accumulator chain). Lp % 128 == 0, Pc % Lp == 0, (N / G) % hs == 0; 16-byte aligned.
+ * (fp32 [G][T Pc][64], summed over the group's heads and the query chunks, hs heads of a chunk to
+ * an accumulator chain). Lp % 128 == 0, Pc % Lp == 0, (N / G) % hs == 0; 16-byte aligned.
  * Errors: FD_ERR_INVALID_ARG, FD_ERR_CUDA; err_dev as for fd_op_linear. */
 fd_status fd_op_attention_bwd(int T, int N, int G, int W, int Pc, int Lp, int L, int hs,
                               const void* q, const void* dO, const void* k, const void* v,

@@ -341,11 +341,11 @@ inline bool gemm_bn_supported(int bn) {
   return bn == 64 || bn == 96 || bn == 128 || bn == 192 || bn == 256;
 }
 // the QKV and GELU epilogues work on 64-column slabs (one head / one 128-byte bf16 row),
-// the fp32 epilogues on 32-column slabs
+// the fp32 epilogues on 32-column slabs. The gated and e4m3 ones store 64-byte rows (64 columns ->
+// 32 bf16 or 64 e4m3, gated e4m3 128 -> 64) and are run and tested at the widths below.
 inline bool gemm_bn_fits_epilogue(int bn, int epi) {
-  if (epi == EPI_SWIGLU) return bn % 128 == 0;  // 128 accumulator columns -> 64 outputs
-  if (epi == EPI_GELU_F8) return bn % 128 == 0;  // 128 e4m3 outputs per 128-byte slab row
-  if (epi == EPI_SWIGLU_F8) return bn % 256 == 0;  // 256 accumulator columns -> 128 outputs
+  if (epi == EPI_SWIGLU || epi == EPI_GELU_F8) return bn % 128 == 0;
+  if (epi == EPI_SWIGLU_F8) return bn % 256 == 0;
   return (epi == EPI_QKV || epi == EPI_GELU) ? bn % 64 == 0 : bn % 32 == 0;
 }
 

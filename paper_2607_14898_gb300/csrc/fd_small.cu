@@ -4,10 +4,10 @@
 //   rmsnorm      h fp32 [M][D] -> bf16(h / sqrt(mean(h^2) + eps) * g)  (pre-norm, Sec. 3.2),
 //                or e4m3 of that times a scale (input of an FP8 MLP)
 //   pixel_head   F fp32 [frames*L][C r_s^2] -> PixelShuffle(r_s) + clamp to [-1, 1], fp32 or
-//                uint8 (Sec. 3.4 "Step 3"); one thread per 4 consecutive output pixels
+//                uint8 (Sec. 3.4 "Step 3"); one thread per 4 consecutive output pixels; in the
+//                decode also chunk counter t += 1 (device-resident, so a captured graph can be
+//                replayed)
 //   kv_append    fp32 K, V of one chunk -> ring slot (K rows bf16, V transposed fp16) (Sec. 3.3)
-//                and, in the decode, chunk counter t += 1 (device-resident, so a captured graph
-//                can be replayed)
 //   chunk_start  a chunk's unshuffle and its temporal RoPE tables in one launch
 //   wait_check   failure-path check: a wait on an mbarrier that nothing arrives at, through
 //                the decode kernels' bounded wait, gives up after a short limit and returns

@@ -7,17 +7,19 @@
 // all T chunks at once: the forward of every block with its activations kept, the L1 term of
 // the pixels, then the backward block by block in reverse. Every product runs on the tensor
 // cores with bf16 operands and fp32 accumulation:
-//   - the linear layers, their input gradients dX = dY W (with the transposed weights) and
-//     weight gradients dW = dY^T X (with transposed activations): the library's GEMM
-//     (gemm_view);
+//   - the linear layers and their input gradients dX = dY W (with the transposed weights): the
+//     library's GEMM (gemm_view, gemm_tup); the weight gradients dW = dY^T X on dY and X as they
+//     are (gemm_wgrad), or on transposed copies of a narrow input (the patch embedding of a
+//     48-channel latent);
 //   - the attention forward: the decode's batched attention kernel with one stream per query
 //     chunk over the window of its key chunks, writing each row's log-sum-exp (attn_fwd);
 //   - the attention backward (fd_attn_bwd.cu): two launches that recompute S = Q K^T and dP =
 //     dO V^T on chip, one for dQ, one for dK and dV.
-// Row-wise and element-wise steps (RMSNorm and its backward, KV-norm / QK-norm with 3D-RoPE and
-// their backward, GELU and GELU', the attention backward's operands, the L1 term through the
-// pixel shuffle, bias and gain sums) are the kernels below. Where a stack's keys per chunk are not a multiple of 8, its
-// attention forward is materialised instead (S, the band softmax, O = P V).
+// Row-wise and element-wise steps (RMSNorm's backward, KV-norm / QK-norm with 3D-RoPE and their
+// backward, GELU and GELU', the L1 term through the pixel shuffle, bias and gain sums) are the
+// kernels of fd_train_rows.cuh; the attention backward's operands and what the materialised
+// attention forward needs are below. That form (S, the band softmax, O = P V) runs where a stack's
+// keys per chunk are not a multiple of 8.
 //
 // Rows: chunk c's L tokens sit at rows c Lp .. c Lp + L - 1 with Lp = 128 ceil(L / 128), the
 // refined frame (c, tau) at rows (c r_t + tau) Lp ...; padding rows carry finite values
@@ -190,7 +192,9 @@ struct fd_trainer_s {
   bf16 *x0, *y16, *yh16, *a1, *vT, *do16, *P16, *dy16, *dyT = nullptr, *xT = nullptr,
       *dqkv16;
   float *z1, *F, *loss_part, *S, *delta, *dq2, *dk2, *dv1, *gA, *gB, *gC, *gtmp = nullptr;
-  int hs = 1;  // heads of one KV group per attention product (a divisor of N / G)
+  // heads of one KV group per product of the materialised attention forward, and per accumulator
+  // chain of dK and dV (a divisor of N / G)
+  int hs = 1;
   float *part_a = nullptr, *part_b = nullptr;  // partial column sums, two sets of part_elems
   size_t part_elems = 0;
   // per-kernel profile (fd_train_profile_enable): events around each launch, by kernel kind
@@ -661,8 +665,10 @@ fd_status fd_train_create(const fd_config* cfg, fd_weights w, int chunks, fd_tra
   const int Mmax = MB > MR ? MB : MR;
   const int Pmax = tr->rt > 1 ? tr->rt * tr->Lp : tr->Lp;
   const int Kmax = std::min(tr->T, tr->Wn) * Pmax;  // keys of one query chunk's window
-  // heads per attention product: all of a KV group's, unless S (fp32 [heads Pmax][Kmax]) would
-  // pass 512 M elements; then the largest divisor of the group size that stays within it
+  // heads per product of the materialised forward: all of a KV group's, unless its S (fp32
+  // [heads Pmax][Kmax]) would pass 512 M elements; then the largest divisor of the group size that
+  // stays within it. The attention backward stores no scores, but adds dK and dV up in chains of
+  // the same heads: they are the sums of the products that it replaced, to the bit.
   {
     const int hpg = tr->N / tr->G;
     tr->hs = 1;

@@ -326,7 +326,8 @@ __device__ __forceinline__ void head_rms(float (&v)[kDh], const float* g, float 
 }
 // One thread does one (row, slot): its 64 values in order, as the sums over a head are. A block
 // stages kQkvBatch rows x up to kQkvSlots slots through shared memory (65 floats per unit: no bank
-// conflicts), so that global memory is read and written in whole lines: a thread reading its own
+// conflicts where a thread walks its own unit; the stores in and the packed reads out of the forward
+// meet 4-way conflicts, the backward's column sums 2-way), so that global memory is read and written in whole lines: a thread reading its own
 // 256 bytes took 136 us forward and 89 us backward on average at 480p, staged 42 and 52. What is left
 // is a block's chain of load, sums and store, so the loads of a batch are issued together (36 / 34
 // us), the four rows of a slot sit in neighbouring threads (a warp then does one kind of slot: 31 /
