@@ -8,12 +8,14 @@
 //               dP^T = V dO^T: dK += dS^T Q, dV += P^T dO over the query blocks (chunks whose
 //               window holds the keys, then the group's heads, then rows)
 //
-// What bounds it: the arithmetic on the scores (about ten instructions an element, 16384 elements
-// a block: ~1300 issue cycles per scheduler against 768 / 1024 tensor cycles), so S and dP are
-// recomputed in both launches (2 of the 5 products twice) rather than stored: writing dS, dS^T
-// and P^T (bf16) and reading them back in N = 64 products moved 12 bytes a score: 45.3 ms of the
-// 480p model's 72.6 ms training step (2 chunks, 24 + 2 blocks); with these kernels the step is
-// 43.8 ms, and its gradients are the same bits.
+// What bounds it: the issue of the arithmetic on the scores. At 480p refinement sizes (2 chunks of
+// 6656 rows, 16 heads on 4 groups) a 128 x 128 block takes 2630 cycles of an SM in either launch: per
+// scheduler 1940 (dK / dV, 15 instructions a score) and 1630 (dQ, 13) issue cycles, against 1024 and
+// 768 of MMA; the FMA pipe is at 50 and 45 %, the transcendental one at 20 %. So S and dP are
+// recomputed in both launches (2 of the 5 products twice) rather than stored: writing dS, dS^T and
+// P^T (bf16) and reading them back in N = 64 products moved 12 bytes a score: 45.3 ms of what was
+// then a 72.6 ms training step of the 480p model (2 chunks, 24 + 2 blocks) and 43.8 ms with these
+// kernels, with the same bits as gradients. They are 9.0 ms of it (24 x 179 us, 2 x 2344 us).
 // Every product's operands are the row-major tiles as they are: K-major for S and dP, and the same
 // shared-memory tile read MN-major (the transpose bit of the instruction descriptor) as B of the
 // gradient products, so nothing is transposed in memory.
