@@ -621,10 +621,21 @@ def op_attention_bwd(q, dO, k, v, lse, delta, W, Lp, L, hs, dq, dk, dv, err=None
                                      _ptr(err), _stream_ptr(stream)), "fd_op_attention_bwd")
 
 
+def _scratch(n, device, stream):
+    """n fp32 elements for a kernel on `stream`, from that stream's own memory: what is given back
+    when the call returns is then only handed out again behind the kernel."""
+    import torch
+    if stream is None:
+        return torch.empty(n, dtype=torch.float32, device=device)
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(_stream_ptr(stream), device=device)
+    with torch.cuda.stream(stream):
+        return torch.empty(n, dtype=torch.float32, device=device)
+
+
 def op_rmsnorm_bwd(x, g, dy, eps, dx, dg, stream=None) -> None:
     M, D = x.shape
-    import torch
-    work = torch.empty(M, D, dtype=torch.float32, device=x.device)
+    work = _scratch(M * D, x.device, stream)
     _check(lib().fd_op_rmsnorm_bwd(_ptr(x), _ptr(g), _ptr(dy), M, D, eps, _ptr(dx), _ptr(dg),
                                    _ptr(work), _stream_ptr(stream)), "fd_op_rmsnorm_bwd")
 
@@ -636,8 +647,7 @@ def op_gelu_bwd(z, da, dz, dz_bf16, stream=None) -> None:
 
 def op_l1_pixel_bwd(F, target, frames, grid_h, grid_w, channels, rs, dF, loss,
                     stream=None) -> None:
-    import torch
-    work = torch.empty((F.numel() + 255) // 256, dtype=torch.float32, device=F.device)
+    work = _scratch((F.numel() + 255) // 256, F.device, stream)
     _check(lib().fd_op_l1_pixel_bwd(_ptr(F), _ptr(target), frames, grid_h, grid_w, channels, rs,
                                     _ptr(dF), _ptr(loss), _ptr(work), _stream_ptr(stream)),
            "fd_op_l1_pixel_bwd")

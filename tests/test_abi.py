@@ -234,3 +234,34 @@ def test_attention_bwd_refuses_shapes_it_cannot_tile():
         assert L.fd_op_attention_bwd(*(c[n] for n in ok), *ptrs) == 1, bad
     ptrs = [ctypes.c_void_p(at + 4)] + [ctypes.c_void_p(at)] * 9 + [None]
     assert L.fd_op_attention_bwd(*ok.values(), *ptrs) == 1  # q off 16 bytes
+
+
+def test_scratch_comes_from_the_stream_it_is_used_on(monkeypatch):
+    """A row-wise op on a stream of the caller's allocates its scratch on that stream, given as a
+    pointer or as an object that holds one: from the current one it would be given back, and handed out again,
+    while the kernel runs."""
+    import contextlib
+    import types
+    torch = pytest.importorskip("torch")
+    current, seen, empty = [None], [], torch.empty
+
+    @contextlib.contextmanager
+    def use(stream):
+        current[0] = stream
+        yield
+        current[0] = None
+
+    def record(*args, **kw):
+        seen.append(current[0])
+        return empty(*args, **kw)
+    ops = types.SimpleNamespace(fd_op_rmsnorm_bwd=lambda *a: 0, fd_op_l1_pixel_bwd=lambda *a: 0)
+    monkeypatch.setattr(fdp, "lib", lambda: ops)
+    monkeypatch.setattr(torch.cuda, "stream", use)
+    monkeypatch.setattr(torch.cuda, "ExternalStream", lambda ptr, device=None: ptr)
+    monkeypatch.setattr(torch, "empty", record)
+    x = torch.zeros(4, 64)
+    for stream, want in ((types.SimpleNamespace(cuda_stream=5), 5), (7, 7)):
+        fdp.op_rmsnorm_bwd(x, x[0], x, 1e-6, x, x[0], stream=stream)
+        fdp.op_l1_pixel_bwd(x, x, 1, 1, 1, 1, 4, x, x[0], stream=stream)
+        assert seen == [want, want]
+        seen.clear()
